@@ -118,23 +118,24 @@ template <int DIM, int AQ = default_aq<DIM>()> __global__ void build_links_kerne
         if (c & CLS_FLOW) L |= 1u << LK::FLOW_SELF;
         if (c & CLS_ADE) L |= 1u << LK::ADE_SELF;
         if (c & CLS_SINK) L |= 1u << LK::SINK;
+        // every link of a blocked node bounces back: its (zero) populations stay where they are
         for (int i = 1; i < F::Q; ++i)
-            if (mask_blocked<DIM>(m, x, y, z, F::c(i, 0), F::c(i, 1), F::c(i, 2), CLS_FLOW)) L |= 1u << i;
+            if ((c & CLS_FLOW) || mask_blocked<DIM>(m, x, y, z, F::c(i, 0), F::c(i, 1), F::c(i, 2), CLS_FLOW)) L |= 1u << i;
         for (int i = 1; i < A::Q; ++i)
-            if (mask_blocked<DIM>(m, x, y, z, A::c(i, 0), A::c(i, 1), A::c(i, 2), CLS_ADE))
+            if ((c & CLS_ADE) || mask_blocked<DIM>(m, x, y, z, A::c(i, 0), A::c(i, 1), A::c(i, 2), CLS_ADE))
                 L |= 1u << (LK::ADE_SELF + i);
         reinterpret_cast<LinkT *>(m.link)[k] = (LinkT)L;
 
         const uint8_t o = m.reset ? (uint8_t)(CLS_FLOW | CLS_ADE) : m.cls_old[q];
         const bool f_open = !(c & CLS_FLOW), a_open = !(c & CLS_ADE);
-        if (f_open && (o & CLS_FLOW)) {  // opens up (or reset): flow at rest
+        if (!f_open || (o & CLS_FLOW)) {  // opens up (or reset): flow at rest; blocked: no populations
             for (int i = 0; i < F::Q; ++i) {
                 if (m.half) reinterpret_cast<__half *>(m.fpop)[i * m.geo.plane + k] = __float2half_rn(0.f);
                 else if (m.dbl) reinterpret_cast<double *>(m.fpop)[i * m.geo.plane + k] = 0.0;
                 else reinterpret_cast<float *>(m.fpop)[i * m.geo.plane + k] = 0.f;
             }
         }
-        if (a_open && (o & CLS_ADE)) {  // opens up (or reset): no substrate
+        if (!a_open || (o & CLS_ADE)) {  // opens up (or reset): no substrate; blocked: no populations
             for (int i = 0; i < A::Q; ++i) {
                 const float v = -A::w(i) * m.c_ref;
                 if (m.half) reinterpret_cast<__half *>(m.gpop)[i * m.geo.plane + k] = __float2half_rn(v);
@@ -208,7 +209,7 @@ __global__ void pop_convert_kernel(const PopArgs a)
                 }
                 a.dense[i * N + q] = v;
             } else {
-                const double dv = a.dense[i * N + q] - a.w[i] * a.offset;
+                const double dv = open ? a.dense[i * N + q] - a.w[i] * a.offset : 0.0;
                 if (a.half) reinterpret_cast<__half *>(a.pop)[p] = __float2half_rn((float)dv);
                 else if (a.dbl) reinterpret_cast<double *>(a.pop)[p] = dv;
                 else reinterpret_cast<float *>(a.pop)[p] = (float)dv;

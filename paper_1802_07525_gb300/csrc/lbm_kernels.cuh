@@ -36,7 +36,15 @@
 
 namespace mfc {
 
-enum : int { MODE_PLAIN = 0, MODE_WRITE = 1, MODE_CHECK = 2 };
+// MODE_SWEEP: several plain steps in one launch (lbm_sweep.cuh).
+enum : int { MODE_PLAIN = 0, MODE_WRITE = 1, MODE_CHECK = 2, MODE_SWEEP = 3 };
+
+// Shape of a sweep launch: one warp per column tile of `width` written columns (even; ntx tiles)
+// and strip of `rows` written rows.
+struct SweepShape {
+    int steps;  // steps per sweep (2 or 3)
+    int ntx, width, rows, strips;
+};
 
 // Pitched layout with a ghost layer (see the file comment).
 struct Geo {

@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include "lbm_pair.cuh"
+#include "lbm_sweep.cuh"
 #include "mfc_internal.h"
 
 #ifndef MFC_DIM
@@ -43,6 +44,16 @@ cudaError_t launch_sink(const Args &a, const StepHost &h, cudaStream_t s)
         if (h.idx32) lbm_step_kernel<D, ST, FLOW, ADE, MODE_PLAIN, AQ, SINK, true><<<grid, h.block, 0, s>>>(a);
         else lbm_step_kernel<D, ST, FLOW, ADE, MODE_PLAIN, AQ, SINK><<<grid, h.block, 0, s>>>(a);
         break;
+    case MODE_SWEEP:
+        if constexpr (D == 2 && !std::is_same<ST, double>::value) {
+            // the rounding of the plain step it stands for
+            constexpr int FORM = FLOW && ADE && AQ == default_aq<D>() && PairedStep<D, ST>::value ? PAIR_FORM : SCALAR_FORM;
+            const dim3 tiles((unsigned)h.sweep.ntx, (unsigned)h.sweep.strips);
+            if (h.sweep.steps == 2) lbm_sweep_kernel<ST, FLOW, ADE, AQ, SINK, FORM, 2><<<tiles, 32, 0, s>>>(a, h.sweep);
+            else lbm_sweep_kernel<ST, FLOW, ADE, AQ, SINK, FORM, SweepSteps<AQ>::value><<<tiles, 32, 0, s>>>(a, h.sweep);
+            break;
+        }
+        return cudaErrorInvalidValue;
     case MODE_WRITE: lbm_step_kernel<D, ST, FLOW, ADE, MODE_WRITE, AQ, SINK><<<grid, h.block, 0, s>>>(a); break;
     default: lbm_step_kernel<D, ST, FLOW, ADE, MODE_CHECK, AQ, SINK><<<grid, h.block, 0, s>>>(a); break;
     }

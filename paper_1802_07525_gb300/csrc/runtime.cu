@@ -11,6 +11,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <chrono>
 #include <new>
 #include <string>
@@ -19,6 +20,7 @@
 
 #include "../../include/mfc.h"
 #include "lbm_aux.cuh"
+#include "lbm_sweep.cuh"
 #include "mfc_internal.h"
 #include "runtime.h"
 
@@ -327,17 +329,57 @@ void mfc::fill_step(const mfc_lattice *L, int kind, int mode, StepHost *h)
 
 namespace {
 
-// Queue one step of `kind` and swap the buffers it wrote; *nblocks receives the blocks (and
-// reduction partials) of the launch.
-mfc_status enqueue_step(mfc_lattice *L, int kind, int mode, int *nblocks = nullptr)
+// Whether plain steps can go several at a time (lbm_sweep.cuh): 2-D, whole, walls across the flow
+// axis, 32-bit offsets.  The others take the one-step kernels.
+bool can_sweep(const mfc_lattice *L)
+{
+    const long long qmax = L->qf > L->qa ? L->qf : L->qa;
+    return L->dim == 2 && !L->dbl && L->offsets32 && qmax * L->geo.plane < (1ll << 31) &&
+           L->desc.bc[1] == MFC_BC_WALL && L->desc.bc[0] != MFC_BC_PERIODIC && !L->desc.cut[0] && !L->desc.cut[1];
+}
+
+// Column tiles and strips of a 2-D sweep of T steps.  The tiles share the columns evenly (even
+// widths).  Strips: as many warps as the GPU holds at once, at least two rows per strip.
+void sweep_shape(const mfc_lattice *L, int T, SweepShape *s)
+{
+    const int widest = T == 2 ? sweep_width<2>() : sweep_width<3>();
+    const int warps = L->qa == 9 ? SweepOccupancy<3, 9>::blocks : SweepOccupancy<2, 5>::blocks;
+    s->steps = T;
+    s->ntx = (L->nx + widest - 1) / widest;
+    s->width = (L->nx + s->ntx - 1) / s->ntx;
+    s->width += s->width & 1;
+    s->ntx = (L->nx + s->width - 1) / s->width;
+    const int want = std::max(1, warps * L->sm_count / s->ntx);
+    s->rows = std::max(2, (L->ny + want - 1) / want);
+    s->strips = (L->ny + s->rows - 1) / s->rows;
+}
+
+// Queue one step of `kind` (`steps` of them for MODE_SWEEP) and swap the buffers it wrote; *nblocks receives
+// the blocks (and reduction partials) of the launch.
+mfc_status enqueue_step(mfc_lattice *L, int kind, int mode, int *nblocks = nullptr, int steps = 1)
 {
     StepHost h;
     fill_step(L, kind, mode, &h);
+    if (mode == MODE_SWEEP) sweep_shape(L, steps, &h.sweep);
     cudaError_t e = launch_step(h, L->stream);
     if (e != cudaSuccess) return fail(L, MFC_ERR_CUDA, std::string("step launch: ") + cudaGetErrorString(e));
     if (nblocks) *nblocks = h.nblocks;
     if (kind != KIND_ADE) L->fcur ^= 1;
     if (kind != KIND_FLOW) L->gcur ^= 1;
+    return MFC_OK;
+}
+
+// Queue n plain steps of `kind`, several at a time where they can go so.
+mfc_status enqueue_plain(mfc_lattice *L, int kind, int n)
+{
+    const int T = !can_sweep(L) ? 1 : (L->qa == 9 ? SweepSteps<9>::value : SweepSteps<5>::value);
+    while (n > 0) {
+        int t = std::min(T, n);
+        if (T == 3 && n == 4) t = 2;  // two and two instead of three and one
+        mfc_status st = t > 1 ? enqueue_step(L, kind, MODE_SWEEP, nullptr, t) : enqueue_step(L, kind, MODE_PLAIN);
+        if (st != MFC_OK) return st;
+        n -= t;
+    }
     return MFC_OK;
 }
 
@@ -358,12 +400,9 @@ mfc_status fill_ghosts(mfc_lattice *L)
 mfc_status enqueue_block(mfc_lattice *L, int kind, int n, bool check)
 {
     int nb = L->nblocks;
-    for (int s = 0; s < n; ++s) {
-        int mode = MODE_PLAIN;
-        if (s == n - 1) mode = check ? MODE_CHECK : MODE_WRITE;
-        mfc_status st = enqueue_step(L, kind, mode, &nb);
-        if (st != MFC_OK) return st;
-    }
+    mfc_status st = enqueue_plain(L, kind, n - 1);
+    if (st == MFC_OK) st = enqueue_step(L, kind, check ? MODE_CHECK : MODE_WRITE, &nb);
+    if (st != MFC_OK) return st;
     if (check) {
         CK(L, launch_finalize(L->partials, nb, L->partials + (size_t)L->max_blocks * NSUM, L->results_d,
                               L->stream));
@@ -379,12 +418,12 @@ void drop_graphs(mfc_lattice *L)
     L->graphs.clear();
 }
 
-// The graph of K steps ending with a check, for the current buffer parity.
-mfc_status graph_for(mfc_lattice *L, int kind, int K, cudaGraphExec_t *out)
+// The graph of K steps ending with a check, for the current buffer parity (a copy of its entry).
+mfc_status graph_for(mfc_lattice *L, int kind, int K, GraphEntry *out)
 {
     for (auto &g : L->graphs)
         if (g.kind == kind && g.K == K && g.fpar == L->fcur && g.gpar == L->gcur) {
-            *out = g.exec;
+            *out = g;
             return MFC_OK;
         }
     const int f0 = L->fcur, g0 = L->gcur;
@@ -392,6 +431,7 @@ mfc_status graph_for(mfc_lattice *L, int kind, int K, cudaGraphExec_t *out)
     mfc_status st = enqueue_block(L, kind, K, true);
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamEndCapture(L->stream, &graph);
+    const int f1 = L->fcur, g1 = L->gcur;
     L->fcur = f0;  // capture recorded the launches; nothing ran
     L->gcur = g0;
     if (st != MFC_OK) {
@@ -403,8 +443,8 @@ mfc_status graph_for(mfc_lattice *L, int kind, int K, cudaGraphExec_t *out)
     e = cudaGraphInstantiate(&exec, graph, 0);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) return fail(L, MFC_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
-    L->graphs.push_back({kind, K, f0, g0, exec});
-    *out = exec;
+    L->graphs.push_back({kind, K, f0, g0, f1, g1, exec});
+    *out = L->graphs.back();
     return MFC_OK;
 }
 
@@ -455,12 +495,12 @@ mfc_status run_phase(mfc_lattice *L, int kind, double tol_flow, double tol_ade, 
         const int n = left >= K ? K : (int)left;
         mfc_status st;
         if (n == K) {
-            cudaGraphExec_t exec;
-            st = graph_for(L, kind, K, &exec);
+            GraphEntry g;
+            st = graph_for(L, kind, K, &g);
             if (st != MFC_OK) return st;
-            CK(L, cudaGraphLaunch(exec, L->stream));
-            if (kind != KIND_ADE && (K & 1)) L->fcur ^= 1;
-            if (kind != KIND_FLOW && (K & 1)) L->gcur ^= 1;
+            CK(L, cudaGraphLaunch(g.exec, L->stream));
+            L->fcur = g.fend;
+            L->gcur = g.gend;
         } else {
             st = enqueue_block(L, kind, n, true);
             if (st != MFC_OK) return st;
@@ -726,6 +766,7 @@ mfc_status mfc::lattice_create(const mfc_lattice_desc *desc, const mfc_params *p
     // transport storage offset: 0, so that the no-substrate start state is stored exactly
     L->c_ref = 0.0f;
     cudaGetDevice(&L->device);
+    cudaDeviceGetAttribute(&L->sm_count, cudaDevAttrMultiProcessorCount, L->device);
     L->block = DEFAULT_BLOCK;
     L->max_blocks = max_launch_blocks(l);
     choose_launch(L);
@@ -879,11 +920,7 @@ static mfc_status step_n(mfc_lattice *L, int kind, int nsteps)
     mfc_status st = enter(L);
     if (st != MFC_OK) return st;
     if (nsteps < 0) return fail(L, MFC_ERR_ARG, "nsteps < 0");
-    for (int s = 0; s < nsteps; ++s) {
-        st = enqueue_step(L, kind, s == nsteps - 1 ? MODE_WRITE : MODE_PLAIN);
-        if (st != MFC_OK) return st;
-    }
-    return MFC_OK;
+    return nsteps ? enqueue_block(L, kind, nsteps, false) : MFC_OK;
 }
 
 MFC_API mfc_status mfc_step_flow(mfc_lattice *L, int nsteps) { return step_n(L, KIND_FLOW, nsteps); }
@@ -895,11 +932,7 @@ MFC_API mfc_status mfc_step_coupled_plain(mfc_lattice *L, int nsteps)
     mfc_status st = enter(L);
     if (st != MFC_OK) return st;
     if (nsteps < 0) return fail(L, MFC_ERR_ARG, "nsteps < 0");
-    for (int s = 0; s < nsteps; ++s) {
-        st = enqueue_step(L, KIND_COUPLED, MODE_PLAIN);
-        if (st != MFC_OK) return st;
-    }
-    return MFC_OK;
+    return enqueue_plain(L, KIND_COUPLED, nsteps);
 }
 
 MFC_API mfc_status mfc_solve_steady(mfc_lattice *L, const mfc_solve_opts *opts, mfc_solve_result *out)

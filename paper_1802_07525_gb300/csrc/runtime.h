@@ -13,7 +13,9 @@
 namespace mfc {
 
 struct GraphEntry {
-    int kind, K, fpar, gpar;
+    int kind, K;
+    int fpar, gpar;  // buffers holding the state before the block
+    int fend, gend;  // and after it
     cudaGraphExec_t exec;
 };
 
@@ -28,7 +30,7 @@ struct mfc_lattice {
     mfc::Geo geo;
     long long N = 0;
     size_t st_bytes = 4;
-    int device = 0;
+    int device = 0, sm_count = 1;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     // stream-ordered pool the device buffers come from (batch instances), or null (cudaMalloc)
