@@ -42,7 +42,8 @@ enum : int { MODE_PLAIN = 0, MODE_WRITE = 1, MODE_CHECK = 2, MODE_SWEEP = 3 };
 // Shape of a sweep launch: one warp per column tile of `width` written columns (even; ntx tiles)
 // and strip of `rows` written rows.
 struct SweepShape {
-    int steps;  // steps per sweep (2 or 3)
+    int steps;  // steps per sweep (2 or 3; up to TILE_STEPS for tiles)
+    int tile;   // tiles of rows exchanging through shared memory, instead of strips
     int ntx, width, rows, strips;
 };
 

@@ -49,6 +49,16 @@ cudaError_t launch_sink(const Args &a, const StepHost &h, cudaStream_t s)
             // the rounding of the plain step it stands for
             constexpr int FORM = FLOW && ADE && AQ == default_aq<D>() && PairedStep<D, ST>::value ? PAIR_FORM : SCALAR_FORM;
             const dim3 tiles((unsigned)h.sweep.ntx, (unsigned)h.sweep.strips);
+            if (h.sweep.tile) {
+                const int warps = h.sweep.rows + 2 * h.sweep.steps;
+                constexpr int row = 2 * TileExchange<FLOW, ADE, AQ>::row * (int)sizeof(float2);
+                auto kernel = lbm_tile_kernel<ST, FLOW, ADE, AQ, SINK, FORM>;
+                const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                           TILE_WARPS * row);
+                if (e != cudaSuccess) return e;
+                kernel<<<tiles, 32 * warps, warps * row, s>>>(a, h.sweep);
+                break;
+            }
             if (h.sweep.steps == 2) lbm_sweep_kernel<ST, FLOW, ADE, AQ, SINK, FORM, 2><<<tiles, 32, 0, s>>>(a, h.sweep);
             else lbm_sweep_kernel<ST, FLOW, ADE, AQ, SINK, FORM, SweepSteps<AQ>::value><<<tiles, 32, 0, s>>>(a, h.sweep);
             break;

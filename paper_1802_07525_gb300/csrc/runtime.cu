@@ -345,6 +345,7 @@ void sweep_shape(const mfc_lattice *L, int T, SweepShape *s)
     const int widest = T == 2 ? sweep_width<2>() : sweep_width<3>();
     const int warps = L->qa == 9 ? SweepOccupancy<3, 9>::blocks : SweepOccupancy<2, 5>::blocks;
     s->steps = T;
+    s->tile = 0;
     s->ntx = (L->nx + widest - 1) / widest;
     s->width = (L->nx + s->ntx - 1) / s->ntx;
     s->width += s->width & 1;
@@ -354,13 +355,81 @@ void sweep_shape(const mfc_lattice *L, int T, SweepShape *s)
     s->strips = (L->ny + s->rows - 1) / s->rows;
 }
 
-// Queue one step of `kind` (`steps` of them for MODE_SWEEP) and swap the buffers it wrote; *nblocks receives
+// Column tiles of a tile launch of T steps, `rows` written rows each (lbm_sweep.cuh).
+void tile_shape(const mfc_lattice *L, int T, int rows, SweepShape *s)
+{
+    const int widest = (64 - ((T + 1) & ~1) - T) & ~1;
+    s->steps = T;
+    s->tile = 1;
+    s->ntx = (L->nx + widest - 1) / widest;
+    s->width = (L->nx + s->ntx - 1) / s->ntx;
+    s->width += s->width & 1;
+    s->ntx = (L->nx + s->width - 1) / s->width;
+    s->rows = rows;
+    s->strips = (L->ny + rows - 1) / rows;
+}
+
+// Estimated time per step, in us, of a tile launch.  Fitted to launches of 8 to 28 warps and 2 to 8 steps
+// on GB300 (FP32 D2Q9 + D2Q5, 128x64 to 1024x512, within 10%): 1.3 us per launch; per block on an SM 71 ns
+// for each row loaded and 48 ns for each row stepped (in proportion to the populations for the other
+// sets); 0.37 us of latency per step, paid once for the blocks that run together and mostly hidden where
+// an SM holds two blocks or more.
+double tile_cost(const mfc_lattice *L, int kind, const SweepShape &s)
+{
+    const double planes = (kind == KIND_ADE ? 0 : 9) + (kind == KIND_FLOW ? 0 : L->qa);
+    const int T = s.steps, warps = s.rows + 2 * T;
+    const double row = planes / 14.0 * (0.048 * T * (s.rows + T - 1) + 0.071 * warps);
+    const double blocks = (double)s.ntx * L->ny / s.rows;  // the last strip's rows beyond the lattice are idle
+    const int per_sm = std::max(1, 32 / warps);            // 64 registers
+    const double n = std::max(1.0, ceil(blocks / L->sm_count));
+    const double rounds = ceil(n / per_sm);
+    const double waits = n <= per_sm ? 1.0 : (per_sm == 1 ? rounds : 0.4 * rounds);
+    return (1.3 + 0.37 * T * waits + n * row) / T;
+}
+
+// The best tile shape for launches of up to `most` steps.
+double best_tile(const mfc_lattice *L, int kind, int most, SweepShape *best)
+{
+    double least = 1e30;
+    for (int T = 2; T <= std::min(most, (int)TILE_STEPS); ++T)
+        for (int rows = 1; rows + 2 * T <= TILE_WARPS; ++rows) {
+            SweepShape s;
+            tile_shape(L, T, rows, &s);
+            const double c = tile_cost(L, kind, s);
+            if (c < least) {
+                least = c;
+                *best = s;
+            }
+        }
+    return least;
+}
+
+// The shape in which the next of n >= 2 plain steps go.  Strips from a million nodes on, where tiles
+// recompute more than they save (2048x1024 FP32: 23.6 against 25.4 us per step, 4096x1024 FP16: 42 against
+// 47; 1024x512: 7.4 against 7.0 and 8.1 against 7.0).  A long run of steps goes in launches of the
+// cheapest tiles, its end in tiles of what is left.
+SweepShape next_sweep(const mfc_lattice *L, int kind, int n)
+{
+    SweepShape s;
+    if (L->N > 1000000) {
+        const int T = L->qa == 9 ? SweepSteps<9>::value : SweepSteps<5>::value;
+        sweep_shape(L, T == 3 && (n == 2 || n == 4) ? 2 : std::min(T, n), &s);
+        return s;
+    }
+    best_tile(L, kind, n, &s);
+    const int launches = (n + s.steps - 1) / s.steps;
+    if (launches * s.steps != n && launches <= 3) best_tile(L, kind, (n + launches - 1) / launches, &s);
+    return s;
+}
+
+// Queue one step of `kind` (MODE_SWEEP: the steps of `shape`) and swap the buffers it wrote; *nblocks receives
 // the blocks (and reduction partials) of the launch.
-mfc_status enqueue_step(mfc_lattice *L, int kind, int mode, int *nblocks = nullptr, int steps = 1)
+mfc_status enqueue_step(mfc_lattice *L, int kind, int mode, int *nblocks = nullptr,
+                        const SweepShape *shape = nullptr)
 {
     StepHost h;
     fill_step(L, kind, mode, &h);
-    if (mode == MODE_SWEEP) sweep_shape(L, steps, &h.sweep);
+    if (shape) h.sweep = *shape;
     cudaError_t e = launch_step(h, L->stream);
     if (e != cudaSuccess) return fail(L, MFC_ERR_CUDA, std::string("step launch: ") + cudaGetErrorString(e));
     if (nblocks) *nblocks = h.nblocks;
@@ -372,13 +441,23 @@ mfc_status enqueue_step(mfc_lattice *L, int kind, int mode, int *nblocks = nullp
 // Queue n plain steps of `kind`, several at a time where they can go so.
 mfc_status enqueue_plain(mfc_lattice *L, int kind, int n)
 {
-    const int T = !can_sweep(L) ? 1 : (L->qa == 9 ? SweepSteps<9>::value : SweepSteps<5>::value);
+    const bool sweep = can_sweep(L);
+    SweepShape s;
+    int shaped_for = 0;  // steps left when s was chosen; it stands until they run short
     while (n > 0) {
-        int t = std::min(T, n);
-        if (T == 3 && n == 4) t = 2;  // two and two instead of three and one
-        mfc_status st = t > 1 ? enqueue_step(L, kind, MODE_SWEEP, nullptr, t) : enqueue_step(L, kind, MODE_PLAIN);
+        mfc_status st;
+        if (sweep && n >= 2) {
+            if (!shaped_for || n < 4 * s.steps) {
+                s = next_sweep(L, kind, n);
+                shaped_for = n;
+            }
+            st = enqueue_step(L, kind, MODE_SWEEP, nullptr, &s);
+            n -= s.steps;
+        } else {
+            st = enqueue_step(L, kind, MODE_PLAIN);
+            n -= 1;
+        }
         if (st != MFC_OK) return st;
-        n -= t;
     }
     return MFC_OK;
 }
