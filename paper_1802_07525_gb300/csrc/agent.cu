@@ -7,7 +7,7 @@
 // per-block shared-memory histograms, then one small kernel that picks the digit).  Spreading
 // moves biomass along chains, one event after another, each event seeing the previous ones, so
 // it runs as a single device thread over the ordered list of cells above the threshold (compacted
-// in order by one block); a walk's path membership is an O(1) mark per node.  Every loop of the
+// in order); a walk's path membership is an O(1) mark per node.  Every loop of the
 // serial kernel is bounded (events by the list, steps by max_walk).
 #include <math.h>
 #include <string.h>
@@ -65,6 +65,8 @@ struct AgentArgs {
     float c_ref;
     unsigned long long *keys;
     int *list, *mark, *path;
+    int *chunk;          // per chunk of LIST_CHUNK nodes: listed nodes, then biofilm nodes
+    double *part_total;  // and biomass
     AgentState *st;
     uint64_t attach_base, spread_base, cycle;
     double c0, cmax, fr, mu, ks;
@@ -148,29 +150,32 @@ __global__ void __launch_bounds__(256) agent_hist_kernel(const unsigned long lon
     if (h[threadIdx.x]) atomicAdd(&st->hist[threadIdx.x], h[threadIdx.x]);
 }
 
-// Fix digit `shift` of the k-th smallest key: the digit whose bucket holds the k_rem-th key.
-__global__ void agent_pick_kernel(AgentState *st, int shift)
+// Fix digit `shift` of the k-th smallest key: the digit whose bucket holds the k_rem-th key.  One block of
+// 256 threads, a scan of the histogram (one thread walking it in global memory took 5 us a digit).
+__global__ void __launch_bounds__(256) agent_pick_kernel(AgentState *st, int shift)
 {
-    if (threadIdx.x == 0 && !st->all) {
-        unsigned int cum = 0;
-        int d = -1;
-        for (int b = 0; b < 256; ++b) {
-            if (cum + st->hist[b] >= st->k_rem) {
-                d = b;
-                break;
-            }
-            cum += st->hist[b];
-        }
-        if (d < 0) {
-            st->all = 1;  // fewer keys than asked for: every front node attaches
-        } else {
-            st->prefix |= (unsigned long long)d << shift;
-            st->mask |= 255ull << shift;
-            st->k_rem -= cum;
-        }
+    __shared__ unsigned int warp_sum[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned int h = st->hist[threadIdx.x], k = st->k_rem;
+    const bool all = st->all != 0;
+    unsigned int incl = h;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
     }
-    __syncthreads();
-    for (int b = threadIdx.x; b < 256; b += blockDim.x) st->hist[b] = 0;
+    if (lane == 31) warp_sum[warp] = incl;
+    __syncthreads();  // every thread has read the state
+    for (int w = 0; w < warp; ++w) incl += warp_sum[w];
+    st->hist[threadIdx.x] = 0;
+    if (all) return;
+    if (incl >= k && incl - h < k) {
+        st->prefix |= (unsigned long long)threadIdx.x << shift;
+        st->mask |= 255ull << shift;
+        st->k_rem = k - (incl - h);
+    } else if (threadIdx.x == 255 && incl < k) {
+        st->all = 1;  // fewer keys than asked for: every front node attaches
+    }
 }
 
 // Attachment, then growth (Eq. 16), node by node.
@@ -199,40 +204,86 @@ __global__ void agent_attach_grow_kernel(const AgentArgs a, int select)
     }
 }
 
-// The nodes above C_max^bio (not electrode), in increasing order: one block, ordered compaction.
-__global__ void __launch_bounds__(1024) agent_list_kernel(const AgentArgs a)
+// The nodes above C_max^bio (not electrode), in increasing order, in three launches: the count in each
+// chunk of LIST_CHUNK nodes, the chunks' offsets (one block), the nodes themselves.  (One block walking
+// the whole lattice took 540 us on 1024x512; these take about 10.)
+constexpr int LIST_CHUNK = 2048;
+
+__device__ __forceinline__ bool agent_listed(const AgentArgs &a, long long q, long long N)
+{
+    return q < N && a.bio[q] > a.cmax && !(a.cls[q] & CLS_ADE);
+}
+
+__global__ void __launch_bounds__(256) agent_list_count_kernel(const AgentArgs a)
+{
+    const long long N = (long long)a.geo.nx * a.geo.ny * a.geo.nz;
+    int n = 0;
+#pragma unroll
+    for (int r = 0; r < LIST_CHUNK / 256; ++r)
+        n += __syncthreads_count(agent_listed(a, (long long)blockIdx.x * LIST_CHUNK + r * 256 + threadIdx.x, N));
+    if (threadIdx.x == 0) a.chunk[blockIdx.x] = n;
+}
+
+// Exclusive scan of the chunk counts, in place.
+__global__ void __launch_bounds__(1024) agent_list_scan_kernel(const AgentArgs a, int chunks)
 {
     __shared__ int warp_off[32];
-    __shared__ int base, chunk;
-    const long long N = (long long)a.geo.nx * a.geo.ny * a.geo.nz;
+    __shared__ int base, total;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) base = 0;
     __syncthreads();
-    for (long long q0 = 0; q0 < N; q0 += blockDim.x) {
-        const long long q = q0 + threadIdx.x;
-        const bool flag = q < N && a.bio[q] > a.cmax && !(a.cls[q] & CLS_ADE);
-        const unsigned int m = __ballot_sync(0xffffffffu, flag);
-        if (lane == 0) warp_off[warp] = __popc(m);
+    for (int c0 = 0; c0 < chunks; c0 += blockDim.x) {
+        const int c = c0 + (int)threadIdx.x;
+        const int v = c < chunks ? a.chunk[c] : 0;
+        int incl = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) warp_off[warp] = incl;
         __syncthreads();
         if (warp == 0) {
-            const int nw = (int)(blockDim.x >> 5);
-            const int v = lane < nw ? warp_off[lane] : 0;
-            int incl = v;
+            int w = warp_off[lane];
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += t;
+                const int t = __shfl_up_sync(0xffffffffu, w, o);
+                if (lane >= o) w += t;
             }
-            if (lane < nw) warp_off[lane] = incl - v;
-            if (lane == 31) chunk = incl;
+            if (lane == 31) total = w;
+            warp_off[lane] = w;
         }
         __syncthreads();
-        if (flag) a.list[base + warp_off[warp] + __popc(m & ((1u << lane) - 1u))] = (int)q;
+        if (c < chunks) a.chunk[c] = base + incl - v + (warp ? warp_off[warp - 1] : 0);
         __syncthreads();
-        if (threadIdx.x == 0) base += chunk;
+        if (threadIdx.x == 0) base += total;
         __syncthreads();
     }
     if (threadIdx.x == 0) a.st->count[ST_NLIST] = (unsigned long long)base;
+}
+
+__global__ void __launch_bounds__(256) agent_list_kernel(const AgentArgs a)
+{
+    __shared__ int warp_off[8];
+    const long long N = (long long)a.geo.nx * a.geo.ny * a.geo.nz;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int at = a.chunk[blockIdx.x];
+    for (int r = 0; r < LIST_CHUNK / 256; ++r) {
+        const long long q = (long long)blockIdx.x * LIST_CHUNK + r * 256 + threadIdx.x;
+        const bool flag = agent_listed(a, q, N);
+        const unsigned int m = __ballot_sync(0xffffffffu, flag);
+        if (lane == 0) warp_off[warp] = __popc(m);
+        __syncthreads();
+        int before = 0, all = 0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            before += w < warp ? warp_off[w] : 0;
+            all += warp_off[w];
+        }
+        if (flag) a.list[at + before + __popc(m & ((1u << lane) - 1u))] = (int)q;
+        at += all;
+        __syncthreads();
+    }
 }
 
 // Spreading: one thread, events in list order.
@@ -305,34 +356,61 @@ template <int DIM> __global__ void agent_spread_kernel(const AgentArgs a)
     a.st->count[ST_STEPS] = steps;
 }
 
-// Classes after the step, and the biofilm statistics (one block, a fixed order of addition).
-__global__ void __launch_bounds__(256) agent_classes_kernel(const AgentArgs a)
+// Classes after the step and the biofilm statistics: one partial per chunk of LIST_CHUNK nodes, then one
+// block adds the partials; the order of addition is fixed.  (One block for all of it took 1.1 ms on
+// 1024x512; these take about 8 us.)
+__device__ __forceinline__ void block_sum_256(double &tot, unsigned long long &nb)
 {
-    const long long N = (long long)a.geo.nx * a.geo.ny * a.geo.nz;
-    double tot = 0.0;
-    unsigned long long nb = 0;
-    for (long long q = threadIdx.x; q < N; q += blockDim.x) {
-        const double b = a.bio[q];
-        const uint8_t c = a.cls[q];
-        a.cls_out[q] = (b > 0.0 && !(c & CLS_ADE)) ? (uint8_t)(CLS_FLOW | CLS_SINK) : c;
-        if (b > 0.0) ++nb;
-        tot += b;
-    }
     __shared__ double sh[256];
     __shared__ unsigned long long sn[256];
     sh[threadIdx.x] = tot;
     sn[threadIdx.x] = nb;
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
+    for (int s = 128; s > 0; s >>= 1) {
         if (threadIdx.x < s) {
             sh[threadIdx.x] += sh[threadIdx.x + s];
             sn[threadIdx.x] += sn[threadIdx.x + s];
         }
         __syncthreads();
     }
+    tot = sh[0];
+    nb = sn[0];
+}
+
+__global__ void __launch_bounds__(256) agent_classes_kernel(const AgentArgs a)
+{
+    const long long N = (long long)a.geo.nx * a.geo.ny * a.geo.nz;
+    double tot = 0.0;
+    unsigned long long nb = 0;
+#pragma unroll
+    for (int r = 0; r < LIST_CHUNK / 256; ++r) {
+        const long long q = (long long)blockIdx.x * LIST_CHUNK + r * 256 + threadIdx.x;
+        if (q >= N) break;
+        const double b = a.bio[q];
+        const uint8_t c = a.cls[q];
+        a.cls_out[q] = (b > 0.0 && !(c & CLS_ADE)) ? (uint8_t)(CLS_FLOW | CLS_SINK) : c;
+        if (b > 0.0) ++nb;
+        tot += b;
+    }
+    block_sum_256(tot, nb);
     if (threadIdx.x == 0) {
-        a.st->total = sh[0];
-        a.st->count[ST_BIOFILM] = sn[0];
+        a.part_total[blockIdx.x] = tot;
+        a.chunk[blockIdx.x] = (int)nb;  // the list's offsets are no longer needed
+    }
+}
+
+__global__ void __launch_bounds__(256) agent_totals_kernel(const AgentArgs a, int chunks)
+{
+    double tot = 0.0;
+    unsigned long long nb = 0;
+    for (int c = threadIdx.x; c < chunks; c += 256) {
+        tot += a.part_total[c];
+        nb += (unsigned long long)a.chunk[c];
+    }
+    block_sum_256(tot, nb);
+    if (threadIdx.x == 0) {
+        a.st->total = tot;
+        a.st->count[ST_BIOFILM] = nb;
     }
 }
 
@@ -354,7 +432,9 @@ mfc_status ensure_agent(mfc_lattice *L, int max_walk)
         L->bytes += bytes;
         return true;
     };
-    if (!get((void **)&L->biomass, N * sizeof(double)) ||
+    const size_t chunks = (N + LIST_CHUNK - 1) / LIST_CHUNK;
+    if (!get((void **)&L->biomass, N * sizeof(double)) || !get((void **)&L->agent_chunk, chunks * sizeof(int)) ||
+        !get((void **)&L->agent_part, chunks * sizeof(double)) ||
         !get((void **)&L->agent_keys, N * sizeof(unsigned long long)) ||
         !get((void **)&L->agent_list, N * sizeof(int)) || !get(&L->agent_state, sizeof(AgentState)))
         return lattice_fail(L, MFC_ERR_OOM, "agent buffers: device allocation failed");
@@ -411,6 +491,8 @@ extern "C" MFC_API mfc_status mfc_agent_step(mfc_lattice *L, const mfc_agent_par
     a.list = L->agent_list;
     a.mark = L->agent_mark;
     a.path = L->agent_path;
+    a.chunk = L->agent_chunk;
+    a.part_total = L->agent_part;
     a.st = static_cast<AgentState *>(L->agent_state);
     a.attach_base = mix64(p->seed ^ ATTACH_TAG);
     a.spread_base = mix64(p->seed ^ SPREAD_TAG ^ (cycle << 32));
@@ -433,10 +515,14 @@ extern "C" MFC_API mfc_status mfc_agent_step(mfc_lattice *L, const mfc_agent_par
         }
     }
     agent_attach_grow_kernel<<<grid_for(N), 256, 0, s>>>(a, p->k_ata > 0 ? 1 : 0);
-    agent_list_kernel<<<1, 1024, 0, s>>>(a);
+    const int chunks = (int)((N + LIST_CHUNK - 1) / LIST_CHUNK);
+    agent_list_count_kernel<<<chunks, 256, 0, s>>>(a);
+    agent_list_scan_kernel<<<1, 1024, 0, s>>>(a, chunks);
+    agent_list_kernel<<<chunks, 256, 0, s>>>(a);
     if (L->dim == 2) agent_spread_kernel<2><<<1, 1, 0, s>>>(a);
     else agent_spread_kernel<3><<<1, 1, 0, s>>>(a);
-    agent_classes_kernel<<<1, 256, 0, s>>>(a);
+    agent_classes_kernel<<<chunks, 256, 0, s>>>(a);
+    agent_totals_kernel<<<1, 256, 0, s>>>(a, chunks);
     ACK(L, cudaGetLastError());
     AgentState host;
     ACK(L, cudaMemcpyAsync(&host, a.st, sizeof host, cudaMemcpyDeviceToHost, s));

@@ -697,6 +697,8 @@ void release(mfc_lattice *L)
     dev_free(L, L->agent_list);
     dev_free(L, L->agent_mark);
     dev_free(L, L->agent_path);
+    dev_free(L, L->agent_chunk);
+    dev_free(L, L->agent_part);
     dev_free(L, L->agent_state);
     if (L->results_h) cudaFreeHost(L->results_h);
     if (L->counts_h) cudaFreeHost(L->counts_h);

@@ -66,6 +66,8 @@ struct mfc_lattice {
     int *agent_mark = nullptr;                // position on the current walk's path, or -1
     int *agent_path = nullptr;                // the walk's path
     int agent_path_cap = 0;
+    int *agent_chunk = nullptr;               // per-chunk counts of the list and of the biofilm
+    double *agent_part = nullptr;             // per-chunk biomass
     void *agent_state = nullptr;              // selection state and counters
 
     std::vector<mfc::GraphEntry> graphs;
