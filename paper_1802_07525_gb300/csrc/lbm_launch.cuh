@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include "lbm_pair.cuh"
+#include "lbm_row.cuh"
 #include "lbm_sweep.cuh"
 #include "mfc_internal.h"
 
@@ -32,17 +33,28 @@ cudaError_t launch_sink(const Args &a, const StepHost &h, cudaStream_t s)
     const dim3 grid((unsigned)h.grid, (unsigned)h.geo.ny, (unsigned)h.geo.nz);
     switch (h.mode) {
     case MODE_PLAIN:
-        // the plain step, the hot loop: 32-bit element offsets where the arrays allow them, and
-        // coupled steps two rows per thread where that was measured faster
-        if constexpr (FLOW && ADE && AQ == default_aq<D>() && PairedStep<D, ST>::value) {
+        // the plain step: 32-bit element offsets where the arrays allow them, and two nodes per thread
+        // where that was measured faster (3-D: along a row; 2-D coupled steps in FP16: in two rows)
+        if constexpr (D == 3 && !std::is_same<ST, double>::value) {
+            if (h.idx32) {
+                constexpr int FORM = FLOW && ADE && std::is_same<ST, __half>::value ? PAIR_FORM : SCALAR_FORM;
+                const int n = (h.geo.nx + 1) / 2;
+                const RowPairs rp = {n, n > 1 ? (uint32_t)(((1ull << 32) + n - 1) / n) : 0u};
+                const dim3 pairs((unsigned)(((long long)n * h.geo.ny + ROW_BLOCK - 1) / ROW_BLOCK), (unsigned)h.geo.nz);
+                lbm_row_kernel<ST, FLOW, ADE, SINK, FORM><<<pairs, ROW_BLOCK, 0, s>>>(a, rp);
+                break;
+            }
+        } else if constexpr (FLOW && ADE && AQ == default_aq<D>() && PairedStep<D, ST>::value) {
             if (h.idx32) {
                 const dim3 pairs((unsigned)h.grid, (unsigned)((h.geo.ny + 1) / 2), (unsigned)h.geo.nz);
                 lbm_pair_kernel<D, ST, SINK><<<pairs, h.block, 0, s>>>(a);
                 break;
             }
+        } else if (h.idx32) {
+            lbm_step_kernel<D, ST, FLOW, ADE, MODE_PLAIN, AQ, SINK, true><<<grid, h.block, 0, s>>>(a);
+            break;
         }
-        if (h.idx32) lbm_step_kernel<D, ST, FLOW, ADE, MODE_PLAIN, AQ, SINK, true><<<grid, h.block, 0, s>>>(a);
-        else lbm_step_kernel<D, ST, FLOW, ADE, MODE_PLAIN, AQ, SINK><<<grid, h.block, 0, s>>>(a);
+        lbm_step_kernel<D, ST, FLOW, ADE, MODE_PLAIN, AQ, SINK><<<grid, h.block, 0, s>>>(a);
         break;
     case MODE_SWEEP:
         if constexpr (D == 2 && !std::is_same<ST, double>::value) {

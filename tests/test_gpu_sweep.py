@@ -96,3 +96,26 @@ def test_2d_sweeps_one_lattice_at_a_time(P, shape, ade_q):
 
 def test_2d_closed_box(P):
     _check(P, (90, 41), 9, bc=(P.MFC_BC_WALL, P.MFC_BC_WALL), tau=0.8, tau_c=0.7, k_sink=1e-3)
+
+
+W, PE, IO = 0, 1, 2  # boundary kinds
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 2), (5, 4, 3), (31, 9, 8), (33, 16, 17), (64, 3, 5), (65, 10, 31)], ids=str)
+@pytest.mark.parametrize("bc", [(W, W, IO), (PE, PE, IO), (W, PE, PE), (W, W, W)], ids=str)
+@pytest.mark.parametrize("prec", ["MFC_FP32", "MFC_FP16_DEV"])
+def test_3d_plain_steps_against_one_node_steps(P, shape, bc, prec):
+    """The two-node plain steps against stored-field steps, which run one node per thread with 64-bit
+    offsets: their multiply-adds may be contracted differently, so 8 steps agree to 2e-6 in FP32 (a few ulp
+    per step on values of order one) and to two FP16 spacings per step in FP16 storage."""
+    kw = dict(precision=getattr(P, prec), bc=bc, tau=0.7, tau_c=0.6, u_in=0.005, k_sink=5e-4, k_half=0.05)
+    a, b = _pair(P, shape, **kw)
+    a.step_coupled_plain(8)
+    for _ in range(8):
+        b.step_coupled(1)
+    for which in (P.MFC_POP_FLOW, P.MFC_POP_ADE):
+        x, y = a.read_populations(which), b.read_populations(which)
+        tol = 2e-6 if prec == "MFC_FP32" else 8 * 2 * 2.0 ** -12
+        assert np.abs(x - y).max() < tol
+    a.close()
+    b.close()
