@@ -45,6 +45,7 @@
 #include <vector>
 
 #include "../../include/mfc.h"
+#include "lbm_row.cuh"
 #include "mfc_internal.h"
 #include "runtime.h"
 
@@ -82,13 +83,21 @@ struct Group {
     size_t arg_bytes = 0;          // size of one argument block (StepArgs of the group)
     void *inst_d = nullptr;        // 2 * slots argument blocks
     uint8_t *inst_h = nullptr;     // pinned staging of the same
-    Tile *tiles_d = nullptr, *tiles_h = nullptr;
+    Tile *tiles_d = nullptr, *tiles_h = nullptr;  // row segments of every instance: check steps, and the
+                                                  // plain steps of those that cannot sweep, which come first
     int tile_cap = 0, ntiles = 0;
-    int *ntiles_d = nullptr, *ntiles_h = nullptr;
+    Tile *fast_d = nullptr, *fast_h = nullptr;    // the other instances' plain steps: tiles of
+                                                  // lbm_batch_tile_kernel, chunks of lbm_batch_row_kernel
+    int fast_cap = 0, nfast = 0, nrest = 0;
+    int *ntiles_d = nullptr, *ntiles_h = nullptr;  // row segments, fast tiles, row segments that cannot sweep
+    int fast_grid = 1;
     int2 *ranges_d = nullptr, *ranges_h = nullptr;  // per slot
     double *partials_d = nullptr;  // NSUM per tile
     int grid = 1;
 };
+
+// What a block steps: 2-D instances in tiles, 3-D ones, 2-D ones that take a launch per step.
+enum { HAS_2D = 1, HAS_3D = 2, HAS_2D_SINGLE = 4 };
 
 enum { SLOT_FREE = 0, SLOT_ACTIVE = 1, SLOT_JOINING = 2, SLOT_RETIRED = 3 };
 
@@ -126,7 +135,7 @@ struct mfc_batch {
     double *results_d = nullptr, *results_h = nullptr;
     std::vector<Slot> slots;
     bool tables_dirty = true;
-    cudaGraphExec_t graphs[1 << NGROUP] = {};
+    cudaGraphExec_t graphs[8] = {};  // per mask of HAS_*
 
     // shared with submitting threads (under mu)
     std::mutex mu;
@@ -176,11 +185,13 @@ void free_group(Group &g)
 {
     cudaFree(g.inst_d);
     cudaFree(g.tiles_d);
+    cudaFree(g.fast_d);
     cudaFree(g.ntiles_d);
     cudaFree(g.ranges_d);
     cudaFree(g.partials_d);
     if (g.inst_h) cudaFreeHost(g.inst_h);
     if (g.tiles_h) cudaFreeHost(g.tiles_h);
+    if (g.fast_h) cudaFreeHost(g.fast_h);
     if (g.ntiles_h) cudaFreeHost(g.ntiles_h);
     if (g.ranges_h) cudaFreeHost(g.ranges_h);
     g = Group();
@@ -277,30 +288,92 @@ mfc_status ensure_tiles(mfc_batch *B, Group &g, int need)
     return MFC_OK;
 }
 
+mfc_status ensure_fast(mfc_batch *B, Group &g, int need)
+{
+    if (need <= g.fast_cap) return MFC_OK;
+    const int cap = std::max(need, 2 * g.fast_cap);
+    BCK(B, cudaStreamSynchronize(B->stream));
+    cudaFree(g.fast_d);
+    if (g.fast_h) cudaFreeHost(g.fast_h);
+    g.fast_d = nullptr;
+    g.fast_h = nullptr;
+    g.fast_cap = 0;
+    BCK(B, cudaMalloc((void **)&g.fast_d, (size_t)cap * sizeof(Tile)));
+    BCK(B, cudaHostAlloc((void **)&g.fast_h, (size_t)cap * sizeof(Tile), cudaHostAllocDefault));
+    g.fast_cap = cap;
+    drop_graphs(B);  // the graphs hold the old table addresses
+    return MFC_OK;
+}
+
+// 2-D instances that go several steps to a launch: walls across the flow axis, no periodic axis.  (In 3-D
+// every instance takes the row kernel.)
+bool can_tile(const mfc_lattice *L)
+{
+    return L->dim == 2 && L->desc.bc[1] == MFC_BC_WALL && L->desc.bc[0] != MFC_BC_PERIODIC;
+}
+
+// Steps and written columns of a 2-D tile launch of this batch.
+int batch_steps(const mfc_batch *B) { return B->half ? BatchSweep<__half>::steps : BatchSweep<float>::steps; }
+
+// The plain steps of a block's 2-D tiles, launch by launch: as equal as they can be, an odd number of
+// launches, so that with the check step every instance is back on buffer A.  n is odd.
+std::vector<int> sweep_plan(const mfc_batch *B, int n)
+{
+    int m = (n + batch_steps(B) - 1) / batch_steps(B);
+    if (!(m & 1)) ++m;
+    std::vector<int> t(m);
+    for (int j = 0; j < m; ++j) t[j] = n / m + (j < n % m ? 1 : 0);
+    return t;
+}
+
+void fast_tiles(const mfc_batch *B, const mfc_lattice *L, int slot, std::vector<Tile> &t)
+{
+    if (L->dim == 2) {
+        const int T = batch_steps(B), rows = BatchSweep<float>::rows;
+        const int widest = (64 - ((T + 1) & ~1) - T) & ~1;
+        const int ntx = (L->nx + widest - 1) / widest;
+        int width = (L->nx + ntx - 1) / ntx;
+        width += width & 1;
+        for (int y = 0; y < L->ny; y += rows)
+            for (int x = 0; x < L->nx; x += width) t.push_back(Tile{slot, x, y, std::min(x + width, L->nx)});
+    } else {
+        const int pairs = row_pairs(L->nx).n * L->ny;
+        for (int z = 0; z < L->nz; ++z)
+            for (int q = 0; q < pairs; q += ROW_BLOCK) t.push_back(Tile{slot, q, 0, z});
+    }
+}
+
 // Tile tables, ranges and argument blocks of the resident instances, uploaded on the stream.
 mfc_status rebuild_tables(mfc_batch *B)
 {
-    std::vector<Tile> tiles[NGROUP];
+    std::vector<Tile> tiles[NGROUP], fast[NGROUP];
+    int nrest[NGROUP] = {};
     for (int gi = 0; gi < NGROUP; ++gi)
         for (int s = 0; s < B->max_slots; ++s) B->grp[gi].ranges_h[s] = make_int2(0, 0);
-    for (int s = 0; s < B->max_slots; ++s) {
-        mfc_lattice *L = B->slots[s].L;
-        if (!L || B->slots[s].state != SLOT_ACTIVE) continue;
-        const int gi = L->dim == 2 ? 0 : 1;
-        Group &g = B->grp[gi];
-        std::vector<Tile> &t = tiles[gi];
-        const int t0 = (int)t.size();
-        for (int z = 0; z < L->nz; ++z)
-            for (int y = 0; y < L->ny; ++y)
-                for (int x0 = 0; x0 < L->nx; x0 += B->block) t.push_back(Tile{s, x0, y, z});
-        g.ranges_h[s] = make_int2(t0, (int)t.size());
-        StepHost h;
-        for (int p = 0; p < 2; ++p) {  // argument blocks of the two buffer parities
-            L->fcur = L->gcur = p;
-            fill_step(L, KIND_COUPLED, MODE_PLAIN, &h);
-            step_args(h, g.inst_h + (size_t)(2 * s + p) * g.arg_bytes);
+    for (int turn = 0; turn < 2; ++turn) {  // first the instances that cannot sweep
+        for (int s = 0; s < B->max_slots; ++s) {
+            mfc_lattice *L = B->slots[s].L;
+            if (!L || B->slots[s].state != SLOT_ACTIVE) continue;
+            const int gi = L->dim == 2 ? 0 : 1;
+            const bool single = L->dim == 2 && !can_tile(L);
+            if (single != (turn == 0)) continue;
+            Group &g = B->grp[gi];
+            std::vector<Tile> &t = tiles[gi];
+            const int t0 = (int)t.size();
+            for (int z = 0; z < L->nz; ++z)
+                for (int y = 0; y < L->ny; ++y)
+                    for (int x0 = 0; x0 < L->nx; x0 += B->block) t.push_back(Tile{s, x0, y, z});
+            g.ranges_h[s] = make_int2(t0, (int)t.size());
+            if (single) nrest[gi] = (int)t.size();
+            else fast_tiles(B, L, s, fast[gi]);
+            StepHost h;
+            for (int p = 0; p < 2; ++p) {  // argument blocks of the two buffer parities
+                L->fcur = L->gcur = p;
+                fill_step(L, KIND_COUPLED, MODE_PLAIN, &h);
+                step_args(h, g.inst_h + (size_t)(2 * s + p) * g.arg_bytes);
+            }
+            L->fcur = L->gcur = 0;
         }
-        L->fcur = L->gcur = 0;
     }
     for (int gi = 0; gi < NGROUP; ++gi) {
         Group &g = B->grp[gi];
@@ -309,9 +382,19 @@ mfc_status rebuild_tables(mfc_batch *B)
         if (st != MFC_OK) return st;
         if (n) memcpy(g.tiles_h, tiles[gi].data(), (size_t)n * sizeof(Tile));
         g.ntiles = n;
-        *g.ntiles_h = n;
+        g.nfast = (int)fast[gi].size();
+        g.nrest = nrest[gi];
+        st = ensure_fast(B, g, std::max(g.nfast, 1));
+        if (st != MFC_OK) return st;
+        if (g.nfast) {
+            memcpy(g.fast_h, fast[gi].data(), (size_t)g.nfast * sizeof(Tile));
+            BCK(B, cudaMemcpyAsync(g.fast_d, g.fast_h, (size_t)g.nfast * sizeof(Tile), cudaMemcpyHostToDevice, B->stream));
+        }
+        g.ntiles_h[0] = n;
+        g.ntiles_h[1] = g.nfast;
+        g.ntiles_h[2] = g.nrest;
         if (n) BCK(B, cudaMemcpyAsync(g.tiles_d, g.tiles_h, (size_t)n * sizeof(Tile), cudaMemcpyHostToDevice, B->stream));
-        BCK(B, cudaMemcpyAsync(g.ntiles_d, g.ntiles_h, sizeof(int), cudaMemcpyHostToDevice, B->stream));
+        BCK(B, cudaMemcpyAsync(g.ntiles_d, g.ntiles_h, 3 * sizeof(int), cudaMemcpyHostToDevice, B->stream));
         BCK(B, cudaMemcpyAsync(g.ranges_d, g.ranges_h, (size_t)B->max_slots * sizeof(int2), cudaMemcpyHostToDevice,
                                B->stream));
         BCK(B, cudaMemcpyAsync(g.inst_d, g.inst_h, (size_t)2 * B->max_slots * g.arg_bytes, cudaMemcpyHostToDevice,
@@ -327,6 +410,7 @@ BatchHost batch_host(const mfc_batch *B, const Group &g, int mode, int parity)
     h.dim = g.dim;
     h.half = B->half;
     h.mode = mode;
+    h.steps = 1;
     h.inst = g.inst_d;
     h.tiles = g.tiles_d;
     h.ntiles = g.ntiles_d;
@@ -337,11 +421,31 @@ BatchHost batch_host(const mfc_batch *B, const Group &g, int mode, int parity)
     return h;
 }
 
+// Plain steps of the instances in the fast table, or of the 2-D ones that cannot sweep.
+BatchHost fast_host(const mfc_batch *B, const Group &g, int steps, int parity)
+{
+    BatchHost h = batch_host(B, g, MODE_SWEEP, parity);
+    h.steps = steps;
+    h.tiles = g.fast_d;
+    h.ntiles = g.ntiles_d + 1;
+    h.grid = g.fast_grid;
+    return h;
+}
+BatchHost rest_host(const mfc_batch *B, const Group &g, int parity)
+{
+    BatchHost h = batch_host(B, g, MODE_PLAIN, parity);
+    h.ntiles = g.ntiles_d + 2;
+    return h;
+}
+
 mfc_status set_block(mfc_batch *B, int block)
 {
     B->block = block;
-    for (int gi = 0; gi < NGROUP; ++gi)
-        B->grp[gi].grid = B->sm_count * batch_occupancy(B->grp[gi].dim, B->half, block);
+    for (int gi = 0; gi < NGROUP; ++gi) {
+        Group &g = B->grp[gi];
+        g.grid = B->sm_count * batch_occupancy(g.dim, B->half, block);
+        g.fast_grid = B->sm_count * (g.dim == 2 ? 2 : (B->half ? RowOccupancy<__half, true>::blocks : RowOccupancy<float, true>::blocks));
+    }
     drop_graphs(B);
     B->tables_dirty = true;
     return rebuild_tables(B);
@@ -382,6 +486,24 @@ mfc_status autotune(mfc_batch *B)
         if (st != MFC_OK) return st;
     }
     if (B->K == 0) {
+        // a step as the blocks take it
+        const int reps = 5;
+        for (int r = -2; r < reps; ++r) {
+            if (r == 0) BCK(B, cudaEventRecord(B->t0, B->stream));
+            for (int gi = 0; gi < NGROUP; ++gi) {
+                const Group &g = B->grp[gi];
+                // as many launches as give every group batch_steps steps
+                for (int k = 0; k < (gi == 0 ? 1 : batch_steps(B)); ++k)
+                    if (g.nfast) BCK(B, launch_batch(fast_host(B, g, gi == 0 ? batch_steps(B) : 1, 0), B->stream));
+                for (int k = 0; k < batch_steps(B); ++k)
+                    if (g.nrest) BCK(B, launch_batch(rest_host(B, g, 0), B->stream));
+            }
+        }
+        BCK(B, cudaEventRecord(B->t1, B->stream));
+        BCK(B, cudaEventSynchronize(B->t1));
+        float ms = 0.f;
+        BCK(B, cudaEventElapsedTime(&ms, B->t0, B->t1));
+        best = ms * 1e-3 / (reps * batch_steps(B));
         // check overhead: the sums of every group, the copy to the host and the host's wait,
         // plus the check step's extra traffic (about 40% of a plain step)
         const double h0 = now_s();
@@ -420,13 +542,21 @@ mfc_status graph_for(mfc_batch *B, int mask, cudaGraphExec_t *out)
     }
     BCK(B, cudaStreamBeginCapture(B->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
-    for (int s = 0; s < B->K && e == cudaSuccess; ++s) {
-        const int mode = s == B->K - 1 ? MODE_CHECK : MODE_PLAIN;
-        for (int gi = 0; gi < NGROUP && e == cudaSuccess; ++gi)
-            if (mask & (1 << gi)) e = launch_batch(batch_host(B, B->grp[gi], mode, s & 1), B->stream);
+    // the plain steps group by group (no group waits for another's results), then the check step of all
+    if (mask & HAS_2D) {
+        const std::vector<int> plan = sweep_plan(B, B->K - 1);
+        for (size_t j = 0; j < plan.size() && e == cudaSuccess; ++j)
+            e = launch_batch(fast_host(B, B->grp[0], plan[j], (int)(j & 1)), B->stream);
     }
+    for (int s = 0; s < B->K - 1 && e == cudaSuccess; ++s) {
+        if (mask & HAS_2D_SINGLE) e = launch_batch(rest_host(B, B->grp[0], s & 1), B->stream);
+        if ((mask & HAS_3D) && e == cudaSuccess) e = launch_batch(fast_host(B, B->grp[1], 1, s & 1), B->stream);
+    }
+    const bool present[NGROUP] = {(mask & (HAS_2D | HAS_2D_SINGLE)) != 0, (mask & HAS_3D) != 0};
+    for (int gi = 0; gi < NGROUP && e == cudaSuccess; ++gi)  // K is even: the last plain step left buffer B
+        if (present[gi]) e = launch_batch(batch_host(B, B->grp[gi], MODE_CHECK, 1), B->stream);
     for (int gi = 0; gi < NGROUP && e == cudaSuccess; ++gi)
-        if (mask & (1 << gi)) {
+        if (present[gi]) {
             batch_finalize_kernel<<<B->max_slots, 256, 0, B->stream>>>(B->grp[gi].ranges_d, B->grp[gi].partials_d,
                                                                        B->results_d);
             e = cudaGetLastError();
@@ -569,7 +699,7 @@ int active_mask(const mfc_batch *B, long long *n_active)
     long long n = 0;
     for (auto &sl : B->slots)
         if (sl.state == SLOT_ACTIVE) {
-            mask |= 1 << (sl.L->dim == 2 ? 0 : 1);
+            mask |= sl.L->dim == 3 ? HAS_3D : (can_tile(sl.L) ? HAS_2D : HAS_2D_SINGLE);
             ++n;
         }
     if (n_active) *n_active = n;
@@ -784,8 +914,8 @@ MFC_API mfc_status mfc_batch_create(const mfc_batch_opts *opts, mfc_batch **out)
         const size_t ib = (size_t)2 * B->max_slots * g.arg_bytes;
         e = cudaMalloc(&g.inst_d, ib);
         if (e == cudaSuccess) e = cudaHostAlloc((void **)&g.inst_h, ib, cudaHostAllocDefault);
-        if (e == cudaSuccess) e = cudaMalloc((void **)&g.ntiles_d, sizeof(int));
-        if (e == cudaSuccess) e = cudaHostAlloc((void **)&g.ntiles_h, sizeof(int), cudaHostAllocDefault);
+        if (e == cudaSuccess) e = cudaMalloc((void **)&g.ntiles_d, 3 * sizeof(int));
+        if (e == cudaSuccess) e = cudaHostAlloc((void **)&g.ntiles_h, 3 * sizeof(int), cudaHostAllocDefault);
         if (e == cudaSuccess) e = cudaMalloc((void **)&g.ranges_d, (size_t)B->max_slots * sizeof(int2));
         if (e == cudaSuccess)
             e = cudaHostAlloc((void **)&g.ranges_h, (size_t)B->max_slots * sizeof(int2), cudaHostAllocDefault);

@@ -32,6 +32,11 @@ template <int DIM, typename ST, bool COUPLED, int AQ, int SINK> struct UuForm {
     static constexpr int outlet_axis = f32 && (!COUPLED || first_order_2d) ? UU_SUM : UU_CHAIN_10;
     static constexpr int outlet_diagonal = f32 && !COUPLED ? UU_SUM : UU_CHAIN_10;
 };
+// Batches (whose kernels choose the consumption at run time) take the reader form of the open boundaries
+// for every storage type.
+template <int DIM, typename ST, int AQ, int SINK> struct ReaderForm {
+    static constexpr bool value = SINK == SINK_RUNTIME || ReaderBoundaries<DIM, ST, AQ>::step;
+};
 template <int DIM, int FORM> __device__ __forceinline__ float2 p_uu(const float2 (&u)[3])
 {
     const float2 m0 = FORM == UU_SUM ? p_rounded_mul(u[0], u[0]) : p_mul(u[0], u[0]);
@@ -165,7 +170,7 @@ __device__ __forceinline__ void collide_ade(float2 (&e)[AdeSet<DIM, AQ>::Q], con
     float2 sink = p_all(0.0f);
     if (sinks) {  // Eq. 16's substrate factor: k C, or k C K_s / (K_s + C)
         sink = p_mul(make_float2(k0, k1), Cs);
-        if constexpr (SINK == SINK_MONOD) {
+        if (SINK == SINK_MONOD || (SINK == SINK_RUNTIME && k_half > 0.0f)) {
             if (k0 != 0.0f) sink.x = sink.x * k_half * recip(k_half + Cs.x);
             if (k1 != 0.0f) sink.y = sink.y * k_half * recip(k_half + Cs.y);
         }

@@ -38,9 +38,8 @@ cudaError_t launch_sink(const Args &a, const StepHost &h, cudaStream_t s)
         if constexpr (D == 3 && !std::is_same<ST, double>::value) {
             if (h.idx32) {
                 constexpr int FORM = FLOW && ADE && std::is_same<ST, __half>::value ? PAIR_FORM : SCALAR_FORM;
-                const int n = (h.geo.nx + 1) / 2;
-                const RowPairs rp = {n, n > 1 ? (uint32_t)(((1ull << 32) + n - 1) / n) : 0u};
-                const dim3 pairs((unsigned)(((long long)n * h.geo.ny + ROW_BLOCK - 1) / ROW_BLOCK), (unsigned)h.geo.nz);
+                const RowPairs rp = row_pairs(h.geo.nx);
+                const dim3 pairs((unsigned)(((long long)rp.n * h.geo.ny + ROW_BLOCK - 1) / ROW_BLOCK), (unsigned)h.geo.nz);
                 lbm_row_kernel<ST, FLOW, ADE, SINK, FORM><<<pairs, ROW_BLOCK, 0, s>>>(a, rp);
                 break;
             }
@@ -143,6 +142,21 @@ size_t MFC_ARGS_FN(const StepHost &h, void *out)
     return sizeof a;
 }
 
+// Plain steps of the instances in the sweep table: several at once in 2-D, one in 3-D.
+template <typename S> cudaError_t launch_batch_sweep(const BatchArgs<2, S> &b, const BatchHost &h, cudaStream_t s)
+{
+    auto kernel = lbm_batch_tile_kernel<S>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BatchSweep<S>::exchange);
+    if (e != cudaSuccess) return e;
+    kernel<<<h.grid, 32 * (BatchSweep<S>::rows + 2 * h.steps), BatchSweep<S>::exchange, s>>>(b, h.steps);
+    return cudaGetLastError();
+}
+template <typename S> cudaError_t launch_batch_sweep(const BatchArgs<3, S> &b, const BatchHost &h, cudaStream_t s)
+{
+    lbm_batch_row_kernel<S><<<h.grid, ROW_BLOCK, 0, s>>>(b);
+    return cudaGetLastError();
+}
+
 // Coupled steps only: a batch advances flow and transport of every instance together.
 cudaError_t MFC_BATCH_FN(const BatchHost &h, cudaStream_t s)
 {
@@ -153,6 +167,8 @@ cudaError_t MFC_BATCH_FN(const BatchHost &h, cudaStream_t s)
     b.partials = h.partials;
     b.parity = h.parity;
     switch (h.mode) {
+    case MODE_SWEEP:
+        return launch_batch_sweep(b, h, s);
     case MODE_PLAIN: lbm_batch_kernel<D, ST, true, true, MODE_PLAIN><<<h.grid, h.block, 0, s>>>(b); break;
     case MODE_WRITE: lbm_batch_kernel<D, ST, true, true, MODE_WRITE><<<h.grid, h.block, 0, s>>>(b); break;
     default: lbm_batch_kernel<D, ST, true, true, MODE_CHECK><<<h.grid, h.block, 0, s>>>(b); break;

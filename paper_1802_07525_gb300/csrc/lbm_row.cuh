@@ -100,12 +100,11 @@ __device__ __forceinline__ void row_store(const StepArgs<3, ST> &a, ST *dst, con
 // Ghost cells of the written flow populations that belong to node (x, y, z) at the inlet or the outlet, from
 // its post-collision populations v and velocity in registers: reading them back after the store costs a
 // round trip to L2 per value, which a small lattice's step waits for.
-template <typename ST, typename FORMS, typename V>
+template <typename ST, typename FORMS, bool WRITER, typename V>
 __device__ __forceinline__ void row_flow_ends(const StepArgs<3, ST> &a, int x, int y, int z, int k, uint32_t L, const V &v,
                                               float u0, float u1, float u2)
 {
     using F = FlowSet<3>;
-    constexpr bool WRITER = !ReaderBoundaries<3, ST>::step;
     const Geo &g = a.geo;
     const int P = (int)g.plane, px = g.px, zs = (int)g.zs;
     if (WRITER && z == 0 && !a.cut[0]) {
@@ -126,22 +125,21 @@ __device__ __forceinline__ void row_flow_ends(const StepArgs<3, ST> &a, int x, i
 }
 
 // The same for the transport populations (v6: the node's population leaving the outlet inwards).
-template <typename ST>
+template <typename ST, bool WRITER>
 __device__ __forceinline__ void row_ade_ends(const StepArgs<3, ST> &a, int z, int k, uint32_t L, float v6)
 {
     const int P = (int)a.geo.plane, zs = (int)a.geo.zs;
-    if (ReaderBoundaries<3, ST>::step) return;
+    if (!WRITER) return;
     if (z == 0 && !a.cut[0] && !((L >> (Links<3>::ADE_SELF + 5)) & 1u)) st(a.gdst + MFC_IDX(5 * P + k - zs, 7 * P), a.gin_dev[5]);
     if (z == a.geo.nz - 1 && !a.cut[1]) st(a.gdst + MFC_IDX(6 * P + k + zs, 7 * P), a.ade_dirichlet ? a.gout_dev[6] : v6);
 }
 
 // Lattices with a periodic axis: the periodic images of node (x, y, z), and the images of the outlet values,
 // read back from the node's stored populations.  SET: the velocity set, Q planes at pop.
-template <typename SET, typename ST, typename FORMS, bool FLOWSET>
+template <typename SET, typename ST, typename FORMS, bool FLOWSET, bool WRITER>
 __device__ __noinline__ void row_images(const StepArgs<3, ST> &a, ST *pop, int x, int y, int z, int k, float u0, float u1,
                                         float u2)
 {
-    constexpr bool WRITER = !ReaderBoundaries<3, ST>::step;
     const Geo &g = a.geo;
     const bool images = on_periodic_boundary<3>(g, a.bc, x, y, z);
     const bool outlet = a.bc[2] == BC_INOUT && z == g.nz - 1 && !a.cut[1] && (FLOWSET || WRITER);
@@ -164,23 +162,21 @@ struct RowPairs {
     uint32_t m;  // ceil(2^32 / n)
 };
 
-// One plain step: grid (pairs of a plane / block, nz); the outlet plane first, whose ghost work is longest.
+// One plain step of pair q (numbered along the rows) of plane z.
 template <typename ST, bool FLOW, bool ADE, int SINK, int FORM>
-__global__ void __launch_bounds__(ROW_BLOCK, RowOccupancy<ST, FLOW && ADE>::blocks) lbm_row_kernel(const StepArgs<3, ST> a, const RowPairs rp)
+__device__ __forceinline__ void row_step(const StepArgs<3, ST> &a, const RowPairs &rp, int q, int z)
 {
     using F = FlowSet<3>;
     using LK = Links<3>;
     using UU = UuForm<3, ST, ADE, 7, SINK>;
-    constexpr bool READER = ReaderBoundaries<3, ST>::step, BOTH = RowOccupancy<ST, FLOW && ADE>::both_sets;
+    constexpr bool READER = ReaderForm<3, ST, 7, SINK>::value, BOTH = RowOccupancy<ST, FLOW && ADE>::both_sets;
     const Geo &g = a.geo;
     const int P = (int)g.plane;
-    const int q = (int)(blockIdx.x * ROW_BLOCK + threadIdx.x);
     int y = rp.n > 1 ? (int)__umulhi((uint32_t)q, rp.m) : q;
     if (y * rp.n > q) --y;
     const bool valid = y < g.ny;
     y = valid ? y : g.ny - 1;  // the last warp's idle lanes repeat the last pair and store nothing
     const int x = valid ? 2 * (q - y * rp.n) : 2 * (rp.n - 1);
-    const int z = blockIdx.y == 0 ? (int)gridDim.y - 1 : (int)blockIdx.y - 1;
     const int k = (int)g.row0 + z * (int)g.zs + y * g.px + x;
     const bool both = x + 1 < g.nx;
     const uint2 L = __ldg(reinterpret_cast<const uint2 *>(a.link + MFC_IDX(k, P - 1)));
@@ -201,12 +197,12 @@ __global__ void __launch_bounds__(ROW_BLOCK, RowOccupancy<ST, FLOW && ADE>::bloc
         if (valid) row_store<F::Q>(a, a.fdst, d, k, both);
         const bool o0 = valid && !(L.x & (1u << LK::FLOW_SELF)), o1 = valid && both && !(L.y & (1u << LK::FLOW_SELF));
         if (ends) {
-            if (o0) row_flow_ends<ST, UU>(a, x, y, z, k, L.x, [&](int i) { return d[i].x; }, u[0].x, u[1].x, u[2].x);
-            if (o1) row_flow_ends<ST, UU>(a, x + 1, y, z, k + 1, L.y, [&](int i) { return d[i].y; }, u[0].y, u[1].y, u[2].y);
+            if (o0) row_flow_ends<ST, UU, !READER>(a, x, y, z, k, L.x, [&](int i) { return d[i].x; }, u[0].x, u[1].x, u[2].x);
+            if (o1) row_flow_ends<ST, UU, !READER>(a, x + 1, y, z, k + 1, L.y, [&](int i) { return d[i].y; }, u[0].y, u[1].y, u[2].y);
         }
         if (periodic) {
-            if (o0) row_images<F, ST, UU, true>(a, a.fdst, x, y, z, k, u[0].x, u[1].x, u[2].x);
-            if (o1) row_images<F, ST, UU, true>(a, a.fdst, x + 1, y, z, k + 1, u[0].y, u[1].y, u[2].y);
+            if (o0) row_images<F, ST, UU, true, !READER>(a, a.fdst, x, y, z, k, u[0].x, u[1].x, u[2].x);
+            if (o1) row_images<F, ST, UU, true, !READER>(a, a.fdst, x + 1, y, z, k + 1, u[0].y, u[1].y, u[2].y);
         }
     }
     if constexpr (ADE) {
@@ -227,13 +223,55 @@ __global__ void __launch_bounds__(ROW_BLOCK, RowOccupancy<ST, FLOW && ADE>::bloc
         if (valid) row_store<7>(a, a.gdst, e, k, both);
         const bool o0 = valid && !(L.x & (1u << LK::ADE_SELF)), o1 = valid && both && !(L.y & (1u << LK::ADE_SELF));
         if (ends) {
-            if (o0) row_ade_ends<ST>(a, z, k, L.x, e[6].x);
-            if (o1) row_ade_ends<ST>(a, z, k + 1, L.y, e[6].y);
+            if (o0) row_ade_ends<ST, !READER>(a, z, k, L.x, e[6].x);
+            if (o1) row_ade_ends<ST, !READER>(a, z, k + 1, L.y, e[6].y);
         }
         if (periodic) {
-            if (o0) row_images<AdeSet<3>, ST, UU, false>(a, a.gdst, x, y, z, k, 0.0f, 0.0f, 0.0f);
-            if (o1) row_images<AdeSet<3>, ST, UU, false>(a, a.gdst, x + 1, y, z, k + 1, 0.0f, 0.0f, 0.0f);
+            if (o0) row_images<AdeSet<3>, ST, UU, false, !READER>(a, a.gdst, x, y, z, k, 0.0f, 0.0f, 0.0f);
+            if (o1) row_images<AdeSet<3>, ST, UU, false, !READER>(a, a.gdst, x + 1, y, z, k + 1, 0.0f, 0.0f, 0.0f);
         }
+    }
+}
+
+// One plain step of a lattice: grid (pairs of a plane / block, nz); the outlet plane first, whose ghost work is
+// longest.
+template <typename ST, bool FLOW, bool ADE, int SINK, int FORM>
+__global__ void __launch_bounds__(ROW_BLOCK, RowOccupancy<ST, FLOW && ADE>::blocks)
+    lbm_row_kernel(const StepArgs<3, ST> a, const RowPairs rp)
+{
+    row_step<ST, FLOW, ADE, SINK, FORM>(a, rp, (int)(blockIdx.x * ROW_BLOCK + threadIdx.x),
+                                        blockIdx.y == 0 ? (int)gridDim.y - 1 : (int)blockIdx.y - 1);
+}
+
+__host__ __device__ __forceinline__ RowPairs row_pairs(int nx)
+{
+    const int n = (nx + 1) / 2;
+    return {n, n > 1 ? (uint32_t)(((1ull << 32) + n - 1) / n) : 0u};
+}
+
+// One plain coupled step of many lattices (batches): a fixed grid walks the table of chunks of ROW_BLOCK pairs
+// (slot, first pair, -, plane); the argument block of a chunk's instance is copied to shared memory.
+template <typename ST>
+__global__ void __launch_bounds__(ROW_BLOCK, RowOccupancy<ST, true>::blocks) lbm_batch_row_kernel(const BatchArgs<3, ST> b)
+{
+    static_assert(sizeof(StepArgs<3, ST>) % 4 == 0, "argument block copied as 32-bit words");
+    __shared__ StepArgs<3, ST> sa;
+    constexpr int WORDS = (int)(sizeof(StepArgs<3, ST>) / 4);
+    const int n = *b.ntiles;
+    int cur = -1;
+    RowPairs rp = {1, 0};
+    for (int t = blockIdx.x; t < n; t += gridDim.x) {
+        const Tile tile = b.tiles[t];
+        if (tile.slot != cur) {  // uniform over the block
+            __syncthreads();     // the previous instance's arguments are no longer read
+            const uint32_t *src = reinterpret_cast<const uint32_t *>(b.inst + 2 * tile.slot + b.parity);
+            uint32_t *dst = reinterpret_cast<uint32_t *>(&sa);
+            for (int w = threadIdx.x; w < WORDS; w += ROW_BLOCK) dst[w] = src[w];
+            __syncthreads();
+            cur = tile.slot;
+            rp = row_pairs(sa.geo.nx);
+        }
+        row_step<ST, true, true, SINK_RUNTIME, SCALAR_FORM>(sa, rp, tile.x0 + (int)threadIdx.x, tile.z);
     }
 }
 

@@ -65,9 +65,9 @@ __device__ __forceinline__ void st_pair(__half *p, float2 v) { *reinterpret_cast
 
 // The inlet or outlet value v as a gathering node sees it: as it is in the reader form, as its
 // ghost cell would keep it in the writer form.
-template <int AQ, typename ST> __device__ __forceinline__ float ghost_value(const ST *tag, float v)
+template <int AQ, int SINK, typename ST> __device__ __forceinline__ float ghost_value(const ST *tag, float v)
 {
-    return ReaderBoundaries<2, ST, AQ>::step ? v : kept(tag, v);
+    return ReaderForm<2, ST, AQ, SINK>::value ? v : kept(tag, v);
 }
 
 // Column state of a lane in tiles that hold the inlet or the outlet.
@@ -92,7 +92,8 @@ template <int AQ, bool FLOW, bool ADE> struct SweepStage {
 
 // Gather the populations along c_i with c_iy < 0 (DOWN: from the row above, `above`) or >= 0 (from
 // the row itself, `own`, and the row below, `below`) of one set into d.
-template <typename ST, int AQ, int Q, bool FLOWSET, bool DOWN, bool EDGE, typename D, typename FB, typename FO, typename FA>
+template <typename ST, int AQ, int SINK, int Q, bool FLOWSET, bool DOWN, bool EDGE, typename D, typename FB, typename FO,
+          typename FA>
 __device__ __forceinline__ void sweep_gather(const StepArgs<2, ST, AQ> &a, D &d, const FB &below, const FO &own,
                                              const FA &above, uint2 L, bool links, const SweepEdge &edge,
                                              float in_down = 0.0f)
@@ -107,14 +108,14 @@ __device__ __forceinline__ void sweep_gather(const StepArgs<2, ST, AQ> &a, D &d,
         const float2 s = cy > 0 ? below(i) : (cy < 0 ? above(i) : own(i));
         d[i] = pull_x(cx, s);
         if (EDGE && !FLOWSET && cx == -1 && edge.last >= 0) {  // outlet: zero gradient, or the Dirichlet value
-            const float v = a.ade_dirichlet ? ghost_value<AQ>(tag, a.gout_dev[i < AQ ? i : 0]) : (edge.last ? s.y : s.x);
+            const float v = a.ade_dirichlet ? ghost_value<AQ, SINK>(tag, a.gout_dev[i < AQ ? i : 0]) : (edge.last ? s.y : s.x);
             if (edge.last) d[i].y = v;
             else d[i].x = v;
         }
         if (EDGE && cx == 1 && edge.inlet) {  // moving-wall bounce-back, or the transport inlet value
-            if constexpr (!FLOWSET) d[i].x = ghost_value<AQ>(tag, a.gin_dev[i < AQ ? i : 0]);
+            if constexpr (!FLOWSET) d[i].x = ghost_value<AQ, SINK>(tag, a.gin_dev[i < AQ ? i : 0]);
             else if constexpr (DOWN) d[i].x = in_down;
-            else d[i].x = ghost_value<AQ>(tag, own(F::opp(i)).x + a.bb_in[i]);
+            else d[i].x = ghost_value<AQ, SINK>(tag, own(F::opp(i)).x + a.bb_in[i]);
         }
     }
     if (links) {
@@ -129,7 +130,7 @@ __device__ __forceinline__ void sweep_gather(const StepArgs<2, ST, AQ> &a, D &d,
 
 // The next row of a stage arrives: v, its populations after the step before, with links L.  The row the
 // stage holds is gathered completely into out (not yet collided); then the stage holds the new row.
-template <typename ST, bool FLOW, bool ADE, int AQ, bool EDGE>
+template <typename ST, bool FLOW, bool ADE, int AQ, int SINK, bool EDGE>
 __device__ __forceinline__ void sweep_arrive(const StepArgs<2, ST, AQ> &a, SweepStage<AQ, FLOW, ADE> &st,
                                              const SweepRow<AQ, FLOW, ADE> &v, uint2 L, const SweepEdge &edge,
                                              SweepRow<AQ, FLOW, ADE> &out)
@@ -143,10 +144,10 @@ __device__ __forceinline__ void sweep_arrive(const StepArgs<2, ST, AQ> &a, Sweep
 #pragma unroll
         for (int i = 0; i < 9; ++i)
             if (F::c(i, 1) >= 0) out.f[i] = st.got.f[i];
-        sweep_gather<ST, AQ, 9, true, true, EDGE>(a, out.f, none, held, now, st.L, st.links, edge, st.in_down);
-        if (EDGE) st.in_down = ghost_value<AQ>((const ST *)nullptr, v.f[6].x + a.bb_in[8]);
+        sweep_gather<ST, AQ, SINK, 9, true, true, EDGE>(a, out.f, none, held, now, st.L, st.links, edge, st.in_down);
+        if (EDGE) st.in_down = ghost_value<AQ, SINK>((const ST *)nullptr, v.f[6].x + a.bb_in[8]);
         st.got.f[0] = v.f[0];
-        sweep_gather<ST, AQ, 9, true, false, EDGE>(a, st.got.f, held, now, none, L, links, edge);
+        sweep_gather<ST, AQ, SINK, 9, true, false, EDGE>(a, st.got.f, held, now, none, L, links, edge);
 #pragma unroll
         for (int i = 1; i < 9; ++i)
             if (F::c(i, 1) > 0) st.up.f[i] = v.f[i];
@@ -158,9 +159,9 @@ __device__ __forceinline__ void sweep_arrive(const StepArgs<2, ST, AQ> &a, Sweep
 #pragma unroll
         for (int i = 0; i < AQ; ++i)
             if (F::c(i, 1) >= 0) out.g[i] = st.got.g[i];
-        sweep_gather<ST, AQ, AQ, false, true, EDGE>(a, out.g, none, held, now, st.L, st.links, edge);
+        sweep_gather<ST, AQ, SINK, AQ, false, true, EDGE>(a, out.g, none, held, now, st.L, st.links, edge);
         st.got.g[0] = v.g[0];
-        sweep_gather<ST, AQ, AQ, false, false, EDGE>(a, st.got.g, held, now, none, L, links, edge);
+        sweep_gather<ST, AQ, SINK, AQ, false, false, EDGE>(a, st.got.g, held, now, none, L, links, edge);
 #pragma unroll
         for (int i = 1; i < AQ; ++i)
             if (F::c(i, 1) > 0) st.up.g[i] = v.g[i];
@@ -230,7 +231,7 @@ __device__ __forceinline__ void sweep_ghosts(const StepArgs<2, ST, AQ> &a, const
     using F = FlowSet<2>;
     using S = AdeSet<2, AQ>;
     using LK = Links<2, AQ>;
-    constexpr bool WRITER = !ReaderBoundaries<2, ST, AQ>::step;
+    constexpr bool WRITER = !ReaderForm<2, ST, AQ, SINK>::value;
     const int P = (int)a.geo.plane, px = a.geo.px;
     if (WRITER && edge.inlet) {
         if constexpr (FLOW) {
@@ -345,7 +346,7 @@ __device__ __forceinline__ void sweep_strip(const StepArgs<2, ST, AQ> &a, int x0
 #pragma unroll
                 for (int i = 0; i < (ADE ? AQ : 0); ++i) v.g[i] = pair_value(in.g[i]);
             }
-            sweep_arrive<ST, FLOW, ADE, AQ, EDGE>(a, st[s], v, L, edge, out);
+            sweep_arrive<ST, FLOW, ADE, AQ, SINK, EDGE>(a, st[s], v, L, edge, out);
             st[s].uf[0] = uf[0];
             st[s].uf[1] = uf[1];
             if (s == 0 && q < q_last) load(in, q + 1);
@@ -502,17 +503,17 @@ __device__ __forceinline__ void tile_steps(const StepArgs<2, ST, AQ> &a, float2 
             auto above = [&](int i) { return above_row[X::place(false, i) * 32]; };
             auto own = [&](int i) { return v.f[i]; };
             d.f[0] = v.f[0];
-            sweep_gather<ST, AQ, 9, true, false, EDGE>(a, d.f, below, own, above, L, links, edge);
-            sweep_gather<ST, AQ, 9, true, true, EDGE>(a, d.f, below, own, above, L, links, edge,
-                                                      EDGE ? ghost_value<AQ>((const ST *)nullptr, v.f[6].x + a.bb_in[8]) : 0.0f);
+            sweep_gather<ST, AQ, SINK, 9, true, false, EDGE>(a, d.f, below, own, above, L, links, edge);
+            sweep_gather<ST, AQ, SINK, 9, true, true, EDGE>(a, d.f, below, own, above, L, links, edge,
+                                                      EDGE ? ghost_value<AQ, SINK>((const ST *)nullptr, v.f[6].x + a.bb_in[8]) : 0.0f);
         }
         if constexpr (ADE) {
             auto below = [&](int i) { return below_row[X::place(true, i) * 32]; };
             auto above = [&](int i) { return above_row[X::place(true, i) * 32]; };
             auto own = [&](int i) { return v.g[i]; };
             d.g[0] = v.g[0];
-            sweep_gather<ST, AQ, AQ, false, false, EDGE>(a, d.g, below, own, above, L, links, edge);
-            sweep_gather<ST, AQ, AQ, false, true, EDGE>(a, d.g, below, own, above, L, links, edge);
+            sweep_gather<ST, AQ, SINK, AQ, false, false, EDGE>(a, d.g, below, own, above, L, links, edge);
+            sweep_gather<ST, AQ, SINK, AQ, false, true, EDGE>(a, d.g, below, own, above, L, links, edge);
         }
         v = d;
         sweep_collide<ST, FLOW, ADE, AQ, SINK, FORM>(a, v, L, links, uf, u);
@@ -555,6 +556,43 @@ __global__ void __launch_bounds__(TILE_WARPS * 32, 1) lbm_tile_kernel(const Step
         tile_steps<ST, FLOW, ADE, AQ, SINK, FORM, true>(a, sh, x0, x1, y0, s.rows, s.steps);
     else
         tile_steps<ST, FLOW, ADE, AQ, SINK, FORM, false>(a, sh, x0, x1, y0, s.rows, s.steps);
+}
+
+// Tiles of many lattices (batches): one launch of T plain steps for every instance that can sweep.  A fixed
+// grid walks the table of tiles; the argument block of a tile's instance is copied to shared memory.  Every
+// launch uses one tile height and the column tiles of BATCH_STEPS steps, so that one table serves launches
+// of any T up to that (measured best for many nodes: FP32 four steps of 8 rows; FP16 three).
+template <typename ST> struct BatchSweep {
+    static constexpr int steps = sizeof(ST) == 4 ? 4 : 3, rows = 8;
+    static constexpr int warps = rows + 2 * steps;
+    static constexpr int exchange = 2 * warps * TileExchange<true, true, 5>::row * (int)sizeof(float2);
+};
+
+template <typename ST>
+__global__ void __launch_bounds__(BatchSweep<ST>::warps * 32, 2) lbm_batch_tile_kernel(const BatchArgs<2, ST> b, int T)
+{
+    static_assert(sizeof(StepArgs<2, ST>) % 4 == 0, "argument block copied as 32-bit words");
+    __shared__ StepArgs<2, ST> sa;
+    extern __shared__ __align__(16) char batch_sh[];
+    float2 *sh = reinterpret_cast<float2 *>(batch_sh);
+    constexpr int WORDS = (int)(sizeof(StepArgs<2, ST>) / 4);
+    const int n = *b.ntiles;
+    int cur = -1;
+    for (int t = blockIdx.x; t < n; t += gridDim.x) {
+        const Tile tile = b.tiles[t];  // x0, first row (y), end of the columns (z)
+        __syncthreads();               // the tile before: its exchange buffers and arguments are no longer read
+        if (tile.slot != cur) {
+            const uint32_t *src = reinterpret_cast<const uint32_t *>(b.inst + 2 * tile.slot + b.parity);
+            uint32_t *dst = reinterpret_cast<uint32_t *>(&sa);
+            for (int w = threadIdx.x; w < WORDS; w += blockDim.x) dst[w] = src[w];
+            __syncthreads();
+            cur = tile.slot;
+        }
+        if (tile.x0 == 0 || tile.x0 + 64 - ((T + 1) & ~1) >= sa.geo.nx)
+            tile_steps<ST, true, true, 5, SINK_RUNTIME, SCALAR_FORM, true>(sa, sh, tile.x0, tile.z, tile.y, BatchSweep<ST>::rows, T);
+        else
+            tile_steps<ST, true, true, 5, SINK_RUNTIME, SCALAR_FORM, false>(sa, sh, tile.x0, tile.z, tile.y, BatchSweep<ST>::rows, T);
+    }
 }
 
 }  // namespace mfc

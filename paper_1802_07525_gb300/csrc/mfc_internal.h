@@ -44,6 +44,7 @@ struct StepHost {
 // One launch of the batch step kernel over a tile table (coupled steps).
 struct BatchHost {
     int dim, half, mode;
+    int steps;          // MODE_SWEEP, 2-D: plain steps of the launch
     const void *inst;   // device array of per-slot argument blocks, two per slot
     const Tile *tiles;  // device tile table
     const int *ntiles;  // device tile count
