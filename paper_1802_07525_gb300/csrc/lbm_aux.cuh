@@ -119,11 +119,22 @@ template <int DIM, int AQ = default_aq<DIM>()> __global__ void build_links_kerne
         if (c & CLS_ADE) L |= 1u << LK::ADE_SELF;
         if (c & CLS_SINK) L |= 1u << LK::SINK;
         // every link of a blocked node bounces back: its (zero) populations stay where they are
-        for (int i = 1; i < F::Q; ++i)
-            if ((c & CLS_FLOW) || mask_blocked<DIM>(m, x, y, z, F::c(i, 0), F::c(i, 1), F::c(i, 2), CLS_FLOW)) L |= 1u << i;
-        for (int i = 1; i < A::Q; ++i)
-            if ((c & CLS_ADE) || mask_blocked<DIM>(m, x, y, z, A::c(i, 0), A::c(i, 1), A::c(i, 2), CLS_ADE))
-                L |= 1u << (LK::ADE_SELF + i);
+        if (x > 0 && x < m.geo.nx - 1 && y > 0 && y < m.geo.ny - 1 && (DIM == 2 || (z > 0 && z < m.geo.nz - 1))) {
+            // inside, a link's source is a node: one class byte serves both sets (the general form below,
+            // for every node, took 640 us on 256x128x128; with this 250)
+#pragma unroll
+            for (int i = 1; i < F::Q; ++i) {
+                const uint8_t o = m.cls_new[q - (F::c(i, 0) + (long long)m.geo.nx * (F::c(i, 1) + (long long)m.geo.ny * F::c(i, 2)))];
+                if ((c | o) & CLS_FLOW) L |= 1u << i;
+                if (i < A::Q && ((c | o) & CLS_ADE)) L |= 1u << (LK::ADE_SELF + i);
+            }
+        } else {
+            for (int i = 1; i < F::Q; ++i)
+                if ((c & CLS_FLOW) || mask_blocked<DIM>(m, x, y, z, F::c(i, 0), F::c(i, 1), F::c(i, 2), CLS_FLOW)) L |= 1u << i;
+            for (int i = 1; i < A::Q; ++i)
+                if ((c & CLS_ADE) || mask_blocked<DIM>(m, x, y, z, A::c(i, 0), A::c(i, 1), A::c(i, 2), CLS_ADE))
+                    L |= 1u << (LK::ADE_SELF + i);
+        }
         reinterpret_cast<LinkT *>(m.link)[k] = (LinkT)L;
 
         const uint8_t o = m.reset ? (uint8_t)(CLS_FLOW | CLS_ADE) : m.cls_old[q];

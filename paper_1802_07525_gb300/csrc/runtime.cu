@@ -3,7 +3,7 @@
 // A lattice owns, on one GPU: two buffers of flow populations and two of transport populations
 // (pull scheme: read one, write the other), one link word per node, the node classes, the
 // FP32 fields (rho - 1, u, C - c_ref) written on check steps, per-block FP64 partial sums and
-// the finalized results (mirrored into pinned host memory).  Steady solves replay a captured
+// the sums (written by the finalize kernel into pinned host memory).  Steady solves replay a captured
 // CUDA graph of K steps (K-1 plain, then one check step that compares the fields with those the
 // previous check stored, stores them and reduces), then read the residuals from the pinned
 // mirror.
@@ -50,9 +50,13 @@ constexpr int FINAL_STAGE1_MAX = 256;
 cudaError_t launch_finalize(const double *partials, int nblocks, double *stage1, double *results,
                             cudaStream_t s)
 {
+    // few partials: one block adds them (two launches cost a small lattice's check 3 us more)
+    if (nblocks <= 2048) {
+        finalize_stage2_kernel<<<1, 256, 0, s>>>(partials, nblocks, results);
+        return cudaGetLastError();
+    }
     int n1 = (nblocks + 63) / 64;
     if (n1 > FINAL_STAGE1_MAX) n1 = FINAL_STAGE1_MAX;
-    if (n1 < 1) n1 = 1;
     finalize_stage1_kernel<<<n1, 256, 0, s>>>(partials, nblocks, stage1);
     finalize_stage2_kernel<<<1, 256, 0, s>>>(stage1, n1, results);
     return cudaGetLastError();
@@ -483,10 +487,9 @@ mfc_status enqueue_block(mfc_lattice *L, int kind, int n, bool check)
     if (st == MFC_OK) st = enqueue_step(L, kind, check ? MODE_CHECK : MODE_WRITE, &nb);
     if (st != MFC_OK) return st;
     if (check) {
-        CK(L, launch_finalize(L->partials, nb, L->partials + (size_t)L->max_blocks * NSUM, L->results_d,
+        // the sums go straight to pinned host memory: the host reads them after waiting for the stream
+        CK(L, launch_finalize(L->partials, nb, L->partials + (size_t)L->max_blocks * NSUM, L->results_h,
                               L->stream));
-        CK(L, cudaMemcpyAsync(L->results_h, L->results_d, sizeof(double) * NRESULT,
-                              cudaMemcpyDeviceToHost, L->stream));
     }
     return MFC_OK;
 }
@@ -686,7 +689,6 @@ void release(mfc_lattice *L)
     dev_free(L, L->fld_u);
     dev_free(L, L->fld_c);
     dev_free(L, L->partials);
-    dev_free(L, L->results_d);
     dev_free(L, L->counts_d);
     dev_free(L, L->staging);
     dev_free(L, L->bounds_err);
@@ -885,7 +887,6 @@ mfc_status mfc::lattice_create(const mfc_lattice_desc *desc, const mfc_params *p
     ok = ok && dalloc(&L->fld_c, (size_t)P * l.fb);
     // per-block partials, then the stage-1 sums of the finalize
     ok = ok && dalloc((void **)&L->partials, ((size_t)L->max_blocks + FINAL_STAGE1_MAX) * NSUM * sizeof(double));
-    ok = ok && dalloc((void **)&L->results_d, NRESULT * sizeof(double));
     ok = ok && dalloc((void **)&L->counts_d, 2 * sizeof(unsigned long long));
 #ifdef MFC_CHECK_BOUNDS
     ok = ok && dalloc((void **)&L->bounds_err, sizeof(unsigned long long));

@@ -44,7 +44,7 @@ struct mfc_lattice {
     // fields (rho - 1, u, C - c_ref): FP32, or FP64 in the FP64 instantiation (dbl)
     void *fld_rho = nullptr, *fld_u = nullptr, *fld_c = nullptr;
     double *partials = nullptr;
-    double *results_d = nullptr, *results_h = nullptr;
+    double *results_h = nullptr;  // pinned: the finalize kernel writes the sums there
     unsigned long long *counts_d = nullptr, *counts_h = nullptr;
     double *staging = nullptr;
     size_t staging_bytes = 0;
