@@ -38,7 +38,7 @@ cudaError_t launch_sink(const Args &a, const StepHost &h, cudaStream_t s)
         if constexpr (D == 3 && !std::is_same<ST, double>::value) {
             if (h.idx32) {
                 constexpr int FORM = FLOW && ADE && std::is_same<ST, __half>::value ? PAIR_FORM : SCALAR_FORM;
-                const RowPairs rp = row_pairs(h.geo.nx);
+                const RowPairs rp = row_pairs(h.geo.nx, h.back);
                 const dim3 pairs((unsigned)(((long long)rp.n * h.geo.ny + ROW_BLOCK - 1) / ROW_BLOCK), (unsigned)h.geo.nz);
                 lbm_row_kernel<ST, FLOW, ADE, SINK, FORM><<<pairs, ROW_BLOCK, 0, s>>>(a, rp);
                 break;

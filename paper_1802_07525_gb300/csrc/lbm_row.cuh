@@ -17,6 +17,11 @@ namespace mfc {
 
 enum : int { ROW_BLOCK = 128 };
 
+// Planes are taken in alternating order (RowPairs::back) where a step reads and writes more than this, three
+// quarters of the L2; below, all of it stays there in any order, and the outlet plane is better taken first
+// (64x40x48 6.04 us per step, 6.16 in turn; 97x71x83 in FP16, 60 MB, the same).
+constexpr long long BACK_BYTES = 96ll << 20;
+
 // Resident blocks per SM.  FP32 coupled steps gather both sets before the first collision (102 registers, 5
 // blocks: 137.4 us per 256x128x128 step, against 141.3 one set after the other at 8 blocks; the one-node
 // kernel took 140); FP16 ones do better with more warps and one set at a time (99.6 us against 104 with
@@ -160,6 +165,11 @@ __device__ __noinline__ void row_images(const StepArgs<3, ST> &a, ST *pop, int x
 struct RowPairs {
     int n;       // pairs per row
     uint32_t m;  // ceil(2^32 / n)
+    // Planes from the last to the first, in every other step: the step before wrote its last planes last, and
+    // reading those first finds them in the L2.  us per step, always upwards and in turn: 97x71x83 27.3 and
+    // 23.4, 128x64x96 30.1 and 27.7, 128x128x128 73.0 and 70.3 (FP16 58.5 and 53.6), 256x128x128 138.1 and
+    // 135.7 (FP16 100.8 and 97.3).  (Loads marked evict-first besides lose more: neighbours' rows share lines.)
+    int back;
 };
 
 // One plain step of pair q (numbered along the rows) of plane z.
@@ -239,14 +249,15 @@ template <typename ST, bool FLOW, bool ADE, int SINK, int FORM>
 __global__ void __launch_bounds__(ROW_BLOCK, RowOccupancy<ST, FLOW && ADE>::blocks)
     lbm_row_kernel(const StepArgs<3, ST> a, const RowPairs rp)
 {
-    row_step<ST, FLOW, ADE, SINK, FORM>(a, rp, (int)(blockIdx.x * ROW_BLOCK + threadIdx.x),
-                                        blockIdx.y == 0 ? (int)gridDim.y - 1 : (int)blockIdx.y - 1);
+    const int z = rp.back ? (int)(gridDim.y - 1 - blockIdx.y) : blockIdx.y == 0 ? (int)gridDim.y - 1 : (int)blockIdx.y - 1;
+    const int b = (int)(rp.back ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
+    row_step<ST, FLOW, ADE, SINK, FORM>(a, rp, b * ROW_BLOCK + (int)threadIdx.x, z);
 }
 
-__host__ __device__ __forceinline__ RowPairs row_pairs(int nx)
+__host__ __device__ __forceinline__ RowPairs row_pairs(int nx, int back = 0)
 {
     const int n = (nx + 1) / 2;
-    return {n, n > 1 ? (uint32_t)(((1ull << 32) + n - 1) / n) : 0u};
+    return {n, n > 1 ? (uint32_t)(((1ull << 32) + n - 1) / n) : 0u, back};
 }
 
 // One plain coupled step of many lattices (batches): a fixed grid walks the table of chunks of ROW_BLOCK pairs
@@ -258,10 +269,12 @@ __global__ void __launch_bounds__(ROW_BLOCK, RowOccupancy<ST, true>::blocks) lbm
     __shared__ StepArgs<3, ST> sa;
     constexpr int WORDS = (int)(sizeof(StepArgs<3, ST>) / 4);
     const int n = *b.ntiles;
+    // the order of RowPairs::back (a mix of 3.4 million nodes, FP32: 83.5 -> 79.0 ms for 800 steps)
+    const bool back = b.parity && n > (int)(BACK_BYTES / (2 * ROW_BLOCK * 26 * 2 * sizeof(ST)));
     int cur = -1;
-    RowPairs rp = {1, 0};
+    RowPairs rp = {1, 0, 0};
     for (int t = blockIdx.x; t < n; t += gridDim.x) {
-        const Tile tile = b.tiles[t];
+        const Tile tile = b.tiles[back ? n - 1 - t : t];
         if (tile.slot != cur) {  // uniform over the block
             __syncthreads();     // the previous instance's arguments are no longer read
             const uint32_t *src = reinterpret_cast<const uint32_t *>(b.inst + 2 * tile.slot + b.parity);

@@ -24,6 +24,7 @@ struct StepHost {
     int nblocks;      // out: blocks of the launch (one reduction partial each)
     int grid, block;  // grid.x (blocks along a row) and threads per block
     SweepShape sweep; // MODE_SWEEP launches
+    int back;         // 3-D plain steps: planes from the last to the first (see RowPairs)
     int idx32;        // every population array has fewer than 2^31 elements: 32-bit offsets
     const void *fsrc;
     void *fdst;

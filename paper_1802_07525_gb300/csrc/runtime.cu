@@ -20,6 +20,7 @@
 
 #include "../../include/mfc.h"
 #include "lbm_aux.cuh"
+#include "lbm_row.cuh"
 #include "lbm_sweep.cuh"
 #include "mfc_internal.h"
 #include "runtime.h"
@@ -277,6 +278,8 @@ void mfc::fill_step(const mfc_lattice *L, int kind, int mode, StepHost *h)
 
     h->grid = L->grid;
     h->block = L->block;
+    const int q = kind == KIND_FLOW ? L->qf : kind == KIND_ADE ? L->qa : L->qf + L->qa;
+    h->back = 2 * q * L->geo.plane * (L->half ? 2 : 4) > BACK_BYTES && (kind == KIND_ADE ? L->gcur : L->fcur);
     // the largest element offset a step forms is below max(Q_flow, Q_transport) planes
     const long long qmax = L->qf > L->qa ? L->qf : L->qa;
     h->idx32 = L->offsets32 && qmax * L->geo.plane < (1ll << 31) ? 1 : 0;

@@ -119,3 +119,33 @@ def test_3d_plain_steps_against_one_node_steps(P, shape, bc, prec):
         assert np.abs(x - y).max() < tol
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("shape,prec", [((97, 71, 83), "MFC_FP32"), ((130, 90, 91), "MFC_FP16_DEV")], ids=str)
+def test_3d_planes_in_alternating_order(P, shape, prec):
+    """Steps that read and write more than the L2 holds take their planes upwards and downwards in turn, a
+    batch its chunks; a single lattice and a batch of it alone round differently by a few FP32 ulp (FP16:
+    storage spacings) per step, so fields agree to 2e-6 (FP16: 5e-3, ten spacings at one)."""
+    kw = dict(tau=0.7, tau_c=0.6, u_in=0.005, k_sink=5e-4)
+    cls = _classes(shape, 3)
+    a, b = (P.Lattice(shape, precision=getattr(P, prec), **kw) for _ in range(2))
+    for g in (a, b):
+        g.set_geometry(cls)
+    a.step_coupled_plain(9)
+    for _ in range(9):
+        b.step_coupled_plain(1)
+    _same(P, a, b)
+    a.close()
+    a = P.Lattice(shape, precision=getattr(P, prec), **kw)
+    a.set_geometry(cls)
+    a.step_coupled(10)
+    batch = P.Batch(check_every=10, precision=getattr(P, prec))
+    ticket = batch.submit(shape, cls, tol_flow=0.0, tol_ade=0.0, max_steps=10, **kw)
+    batch.run()
+    got = batch.poll(ticket)
+    batch.close()
+    tol = 2e-6 if prec == "MFC_FP32" else 5e-3
+    for x, y in zip((got["u"], got["c"]), a.read_fields()[1:3]):
+        assert np.abs(x - y).max() < tol
+    a.close()
+    b.close()
