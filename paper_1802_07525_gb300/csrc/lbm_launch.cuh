@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include "lbm_pair.cuh"
+#include "lbm_march.cuh"
 #include "lbm_row.cuh"
 #include "lbm_sweep.cuh"
 #include "mfc_internal.h"
@@ -72,6 +73,16 @@ cudaError_t launch_sink(const Args &a, const StepHost &h, cudaStream_t s)
             }
             if (h.sweep.steps == 2) lbm_sweep_kernel<ST, FLOW, ADE, AQ, SINK, FORM, 2><<<tiles, 32, 0, s>>>(a, h.sweep);
             else lbm_sweep_kernel<ST, FLOW, ADE, AQ, SINK, FORM, SweepSteps<AQ>::value><<<tiles, 32, 0, s>>>(a, h.sweep);
+            break;
+        }
+        if constexpr (D == 3 && std::is_same<ST, float>::value && FLOW && ADE) {
+            static_assert(!ReaderBoundaries<3, float>::step, "step 1 reads the ghost cells of the writer form");
+            auto kernel = lbm_march_kernel<SINK>;
+            const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MarchExchange::bytes);
+            if (e != cudaSuccess) return e;
+            const dim3 columns((unsigned)h.sweep.ntx, (unsigned)((h.geo.ny + MARCH_ROWS - 3) / (MARCH_ROWS - 2)),
+                               (unsigned)h.sweep.strips);
+            kernel<<<columns, MARCH_ROWS * 32, MarchExchange::bytes, s>>>(a, h.sweep);
             break;
         }
         return cudaErrorInvalidValue;

@@ -20,7 +20,7 @@
 
 #include "../../include/mfc.h"
 #include "lbm_aux.cuh"
-#include "lbm_row.cuh"
+#include "lbm_march.cuh"
 #include "lbm_sweep.cuh"
 #include "mfc_internal.h"
 #include "runtime.h"
@@ -336,13 +336,16 @@ void mfc::fill_step(const mfc_lattice *L, int kind, int mode, StepHost *h)
 
 namespace {
 
-// Whether plain steps can go several at a time (lbm_sweep.cuh): 2-D, whole, walls across the flow
-// axis, 32-bit offsets.  The others take the one-step kernels.
-bool can_sweep(const mfc_lattice *L)
+// Whether plain steps can go several at a time (lbm_sweep.cuh, lbm_march.cuh): whole lattices with walls
+// across the flow axis, 32-bit offsets.  The others take the one-step kernels.
+bool can_sweep(const mfc_lattice *L, int kind)
 {
+    if (L->dim == 3 && (kind != KIND_COUPLED || L->half)) return false;
     const long long qmax = L->qf > L->qa ? L->qf : L->qa;
-    return L->dim == 2 && !L->dbl && L->offsets32 && qmax * L->geo.plane < (1ll << 31) &&
-           L->desc.bc[1] == MFC_BC_WALL && L->desc.bc[0] != MFC_BC_PERIODIC && !L->desc.cut[0] && !L->desc.cut[1];
+    const int fa = L->dim == 2 ? 0 : 2;
+    for (int ax = 0; ax < L->dim; ++ax)
+        if (L->desc.bc[ax] == MFC_BC_PERIODIC || (ax != fa && L->desc.bc[ax] != MFC_BC_WALL)) return false;
+    return !L->dbl && L->offsets32 && qmax * L->geo.plane < (1ll << 31) && !L->desc.cut[0] && !L->desc.cut[1];
 }
 
 // Column tiles and strips of a 2-D sweep of T steps.  The tiles share the columns evenly (even
@@ -411,6 +414,36 @@ double best_tile(const mfc_lattice *L, int kind, int most, SweepShape *best)
     return least;
 }
 
+// Columns of a 3-D sweep of two steps: even column tiles, and as many pieces along z as make the last round
+// of blocks (one per SM) full, counting two turns more than planes for each.  Returns whether it is faster
+// than two one-step launches: a turn takes 1.32 us per step (1.24 to 1.49 over 21 lattices of 64x40x48 to
+// 300x200x150), the row kernel at least 0.0323 ns per node, so from 41000 nodes per turn on.  us per step, march
+// against row: 120x120x120 53.3 and 57.4, 200x150x100 93.9 and 98.3, 256x128x128 134.3 and 135.7, 256x256x128
+// 250 and 268; 97x71x83 22.9 and 23.4 (taken as even); below the line, 128x128x128 83 and 70, 128x64x96 34.8
+// and 27.7, 64x40x48 9.8 and 6.0.
+bool march_shape(const mfc_lattice *L, SweepShape *s)
+{
+    s->steps = 2;
+    s->tile = 0;
+    s->ntx = (L->nx + MARCH_WIDTH - 1) / MARCH_WIDTH;
+    s->width = (L->nx + s->ntx - 1) / s->ntx;
+    s->width += s->width & 1;
+    s->ntx = (L->nx + s->width - 1) / s->width;
+    const long long tiles = (long long)s->ntx * ((L->ny + MARCH_ROWS - 3) / (MARCH_ROWS - 2));
+    long long least = -1;
+    for (int planes = 1; planes <= L->nz; ++planes) {
+        const int strips = (L->nz + planes - 1) / planes;
+        const long long rounds = (tiles * strips + L->sm_count - 1) / L->sm_count;
+        const long long turns = rounds * (planes + 2);
+        if (least < 0 || turns <= least) {
+            least = turns;
+            s->rows = planes;
+            s->strips = strips;
+        }
+    }
+    return L->N > 41000 * least;
+}
+
 // The shape in which the next of n >= 2 plain steps go.  Strips from a million nodes on, where tiles
 // recompute more than they save (2048x1024 FP32: 23.6 against 25.4 us per step, 4096x1024 FP16: 42 against
 // 47; 1024x512: 7.4 against 7.0 and 8.1 against 7.0).  A long run of steps goes in launches of the
@@ -418,6 +451,10 @@ double best_tile(const mfc_lattice *L, int kind, int most, SweepShape *best)
 SweepShape next_sweep(const mfc_lattice *L, int kind, int n)
 {
     SweepShape s;
+    if (L->dim == 3) {
+        march_shape(L, &s);
+        return s;
+    }
     if (L->N > 1000000) {
         const int T = L->qa == 9 ? SweepSteps<9>::value : SweepSteps<5>::value;
         sweep_shape(L, T == 3 && (n == 2 || n == 4) ? 2 : std::min(T, n), &s);
@@ -448,8 +485,8 @@ mfc_status enqueue_step(mfc_lattice *L, int kind, int mode, int *nblocks = nullp
 // Queue n plain steps of `kind`, several at a time where they can go so.
 mfc_status enqueue_plain(mfc_lattice *L, int kind, int n)
 {
-    const bool sweep = can_sweep(L);
     SweepShape s;
+    const bool sweep = n >= 2 && can_sweep(L, kind) && (L->dim == 2 || march_shape(L, &s));
     int shaped_for = 0;  // steps left when s was chosen; it stands until they run short
     while (n > 0) {
         mfc_status st;

@@ -149,3 +149,11 @@ def test_3d_planes_in_alternating_order(P, shape, prec):
         assert np.abs(x - y).max() < tol
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("shape", [(60, 114, 64), (119, 119, 120), (120, 113, 67)], ids=str)
+@pytest.mark.parametrize("bc,k_half,outlet", [((W, W, IO), 0.0, 0), ((W, W, IO), 0.05, 1), ((W, W, W), 0.0, 0)], ids=str)
+def test_3d_two_steps_per_launch(P, shape, bc, k_half, outlet):
+    """Lattices whose coupled steps go two at a time, against one step per launch: exact."""
+    _check(P, shape, 5, bc=bc, tau=0.7, tau_c=0.6, u_in=0.005, k_sink=5e-4, k_half=k_half, ade_outlet=outlet,
+           c_out=0.3, u_scale=1.25)
