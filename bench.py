@@ -440,10 +440,10 @@ def traffic_record(kernel):
 # ---- GPU legs --------------------------------------------------------------------------------
 
 def time_plain_steps(P, lat, stream, M=400):
-    """Average duration of the plain fused step kernel, in ms, two ways, each bracketed by CUDA
+    """Average duration of a plain fused step, in ms, two ways, each bracketed by CUDA
     events on the lattice stream: (1) launched as mfc_solve_steady launches it, one CUDA graph of
-    M steps (M - 1 plain steps and one check step, then the two sum kernels), the block's time
-    over M: an upper bound on the plain launch's duration, since the rest takes longer than a
+    M steps (M - 1 plain steps, several per launch where they can, and one check step, then the sums),
+    the block's time over M: an upper bound on the plain step, since the rest takes longer than a
     plain step; (2) M direct launches (mfc_step_coupled), which adds each launch's gap."""
     import torch
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -462,6 +462,18 @@ def time_plain_steps(P, lat, stream, M=400):
     return graph_ms, e0.elapsed_time(e1) / M
 
 
+def plain_kernel(dim, prec_bytes, nodes, ade_q=0):
+    """The kernel that long runs of plain steps of a bench workload take, and the steps that it carries per
+    launch: in 2-D strips of two (D2Q9 transport: three) from a million nodes on, below that tiles of up to
+    eight; in 3-D two steps per launch in FP32 at the electrode's size, else one."""
+    t = "half" if prec_bytes == 2 else "float"
+    if dim == 2:
+        if nodes > 1000000:
+            return "lbm_sweep_kernel<%s,d2q%d>" % (t, ade_q or 5), 3 if ade_q == 9 else 2
+        return "lbm_tile_kernel<%s>" % t, 8
+    return ("lbm_march_kernel", 2) if prec_bytes == 4 else ("lbm_row_kernel<half>", 1)
+
+
 def step_bytes(dim, prec_bytes, flow_open, ade_open, ade_q=0):
     """Algorithmic bytes of one fused step: every population of every open node read once and
     written once."""
@@ -474,7 +486,7 @@ def step_bytes(dim, prec_bytes, flow_open, ade_open, ade_q=0):
 def leg_variants(P, peak):
     """The 2048x1024 anode in FP32, the FP16-storage 2-D step, the D2Q9 transport, the
     saturating consumption of Eq. 16 and the 3-D electrode in FP32 and FP16: MLUPS over graph
-    blocks and the plain kernel's fraction of the HBM roofline."""
+    blocks and the plain kernel's fraction of the HBM roofline (bytes of a launch over its time)."""
     import torch
     import mfc_inputs as mi
     out = {}
@@ -510,10 +522,12 @@ def leg_variants(P, peak):
         lat.set_launch(block=lat.get_launch()["block"], offsets32=1)
         sb = 2 if prec == P.MFC_FP16_DEV else 4
         byt = step_bytes(w.dim, sb, fo, ao, aq)
-        ach = byt / (kern_ms * 1e-3) / 1e9
+        kname, spl = plain_kernel(w.dim, sb, w.nodes, aq)
+        ach = byt / (spl * kern_ms * 1e-3) / 1e9
         out[name] = {"mlups": w.nodes * steps / (ms * 1e-3) / 1e6, "steps": steps,
                      "kernel_ms": kern_ms, "kernel_ms_direct": kern_direct_ms,
                      "kernel_ms_offsets64": kern64_ms,
+                     "kernel": kname, "steps_per_launch": spl,
                      "algorithmic_bytes_per_launch": byt,
                      "achieved_gbs": ach, "roofline_frac": ach / peak,
                      "bytes_per_node": byt / w.nodes}
@@ -857,10 +871,9 @@ def main():
     working_set = 2 * sb * (qf + qa) * w.nodes
     bytes_per_launch = step_bytes(w.dim, sb, flow_open, ade_open)
     peak, peak_kind = measured_peaks()
-    achieved = bytes_per_launch / (kern_ms * 1e-3) / 1e9
-    # FP16 storage steps two rows per thread with paired FP32 arithmetic (lbm_pair_kernel)
-    kname = ("lbm_pair_kernel<%d,half,0>" % w.dim if sb == 2 else
-             "lbm_step_kernel<%d,float,true,true,0>" % w.dim)
+    kname, spl = plain_kernel(w.dim, sb, w.nodes)
+    # a launch of several steps reads and writes every population once
+    achieved = bytes_per_launch / (spl * kern_ms * 1e-3) / 1e9
     traffic = traffic_record(kname)
 
     # end to end through the public API with host buffers: upload classes from pinned memory,
@@ -924,8 +937,9 @@ def main():
 
     if rank == 0:
         nblocks = (args.steps + K - 1) // K
-        # per block: K step kernels and the two sum kernels
-        launches = args.steps + 2 * nblocks
+        # per block: the plain steps' launches, the check step and the sums (two kernels from 2048
+        # partials on, one per 256 nodes)
+        launches = nblocks * ((K - 1 + spl - 1) // spl + 1 + (2 if w.nodes > 2048 * 256 else 1))
         line = {
             "metric": METRIC, "value": value, "unit": "MLUPS", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms / args.steps,
@@ -942,10 +956,10 @@ def main():
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic,
                          "peak_source": f"{peak_kind} hbm_gbs",
-                         "kernel": kname, "kernel_ms": kern_ms,
+                         "kernel": kname, "kernel_ms": kern_ms, "steps_per_launch": spl,
                          "kernel_ms_timing": "mean step of a 400-step CUDA graph as mfc_solve_steady "
-                                             "runs it (399 plain steps, 1 check step, 2 sum kernels): "
-                                             "an upper bound on the plain launch",
+                                             "runs it (399 plain steps, 1 check step, the sums): "
+                                             "an upper bound on a plain step's share of its launch",
                          "kernel_ms_direct": kern_direct_ms,
                          "algorithmic_bytes_per_launch": bytes_per_launch},
             "cpu_baseline": cpu,

@@ -4,9 +4,11 @@
 // Requests wait in a first-come-first-served queue and are admitted while an instance slot is
 // free and the request's device memory fits the budget.  An admitted request becomes a lattice
 // (mfc_lattice) whose buffers come from the batch's stream-ordered memory pool.  All active
-// instances of one dimension advance in one launch per step: a fixed grid (resident blocks per
-// SM x SMs) walks a tile table listing every row segment of every instance, instance after
-// instance (lbm_batch_kernel).  A block is a CUDA graph of K steps (K - 1 plain, one check) per
+// instances of one dimension advance together: a fixed grid (resident blocks per SM x SMs) walks a
+// tile table that lists every tile of every instance, instance after instance.  Plain steps of 2-D
+// instances with walls across the flow go several per launch (lbm_batch_tile_kernel), 3-D ones two
+// nodes per thread (lbm_batch_row_kernel); check steps, and plain steps of the other 2-D instances, walk row
+// segments (lbm_batch_kernel).  A block is a CUDA graph of K steps (K - 1 plain, one check) per
 // group of dimensions present, the per-instance FP64 sums over each instance's tiles, and one
 // copy of all instances' sums to pinned host memory.
 //

@@ -424,14 +424,12 @@ __device__ __forceinline__ bool tile_on_open_boundary(const Geo &g, const int (&
 // than at 32), FP32 2-D steps with D2Q9 transport, and 2-D store/check steps 40.  3-D steps are
 // latency-bound and gain from warps: FP32 with 5 blocks of 256 threads (51 registers: 148 us per
 // 256x128x128 step, against 211 us uncapped at 128 registers) and FP16 with 4 (64 registers:
-// 154 against 178 us); tighter caps spill and run slower.  With 32-bit offsets the FP16 3-D plain
-// step fits 48 registers without spills, and 5 blocks run it 6% faster (119.0 against 126.8 us);
-// the FP32 3-D one gains nothing from 6 blocks (138.9 against 139.5 us, with spills).  The FP64
-// instantiation (a parity reference, twice the registers per value) gets 128.
-template <int DIM, int MODE, typename ST = float, int AQ = default_aq<DIM>(), bool IDX32 = false>
+// 154 against 178 us); tighter caps spill and run slower.  (Plain 3-D steps with 32-bit offsets run
+// two nodes per thread, lbm_row.cuh.)  The FP64 instantiation (a parity reference, twice the
+// registers per value) gets 128.
+template <int DIM, int MODE, typename ST = float, int AQ = default_aq<DIM>()>
 struct StepOccupancy {
     static constexpr int blocks =
-        (IDX32 && MODE == MODE_PLAIN && DIM == 3 && sizeof(ST) == 2) ? 5 :
         sizeof(ST) == 8 ? 2
                         : (DIM == 2 ? ((MODE == MODE_PLAIN && sizeof(ST) == 4 && AQ == 5) ? 8 : 6)
                                     : (sizeof(ST) == 4 ? 5 : 4));
@@ -692,7 +690,7 @@ __device__ __forceinline__ void step_node(const StepArgs<DIM, ST, AQ> &a, int x0
 // partial per block on check steps.
 template <int DIM, typename ST, bool FLOW, bool ADE, int MODE, int AQ = default_aq<DIM>(), int SINK = SINK_LINEAR,
           bool IDX32 = false>
-__global__ void __launch_bounds__(256, StepOccupancy<DIM, MODE, ST, AQ, IDX32>::blocks) lbm_step_kernel(const StepArgs<DIM, ST, AQ> a)
+__global__ void __launch_bounds__(256, StepOccupancy<DIM, MODE, ST, AQ>::blocks) lbm_step_kernel(const StepArgs<DIM, ST, AQ> a)
 {
     using IX = typename std::conditional<IDX32, int, long long>::type;
     using R = ArithT<ST>;

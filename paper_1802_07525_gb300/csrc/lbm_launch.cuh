@@ -34,7 +34,7 @@ cudaError_t launch_sink(const Args &a, const StepHost &h, cudaStream_t s)
     const dim3 grid((unsigned)h.grid, (unsigned)h.geo.ny, (unsigned)h.geo.nz);
     switch (h.mode) {
     case MODE_PLAIN:
-        // the plain step: 32-bit element offsets where the arrays allow them, and two nodes per thread
+        // one plain step: 32-bit element offsets where the arrays allow them, and two nodes per thread
         // where that was measured faster (3-D: along a row; 2-D coupled steps in FP16: in two rows)
         if constexpr (D == 3 && !std::is_same<ST, double>::value) {
             if (h.idx32) {

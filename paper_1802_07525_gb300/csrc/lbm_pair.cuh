@@ -1,4 +1,4 @@
-// Plain coupled steps with two nodes per thread: node (x, y, z) and (x, y + 1, z), the same
+// 2-D plain coupled steps in FP16 with two nodes per thread: node (x, y) and (x, y + 1), the same
 // stream-collide as step_node (Eqs. 4, 5, 9-13 with the bounce-back of Eq. 11), with the
 // collision of both nodes carried out by Blackwell's paired FP32 instructions (one FFMA2, FADD2 or
 // FMUL2 for the two lanes).  In FP16 storage the single-node step spends its issue slots on
@@ -6,12 +6,14 @@
 // FP32); pairing halves the collision's instructions and gives every thread twice the loads in
 // flight.  Loads, stores, link bits and boundary work stay per node.
 //
-// Pairs run along y, never along the inlet/outlet axis (x in 2-D, z in 3-D), so the inlet and
+// Pairs run along y, never along the inlet/outlet axis, so the inlet and
 // outlet tests are the same for both nodes of a pair.  Every lane rounds as an FP32 instruction
 // does, but the operations are grouped differently from step_node's (the equilibrium is formed as
 // w (1 + rho') t + w rho', the momentum as the sum over c = +1 less the sum over c = -1), so the
-// two forms agree to FP32 rounding, not bit for bit.  Only plain steps use the pairs; check steps
-// and stored-field steps stay on step_node, which reads and writes the same buffers.
+// two forms agree to FP32 rounding, not bit for bit.  Single plain steps use the pairs (and lattices
+// whose steps cannot go several per launch: a periodic axis, a cut face); lbm_sweep.cuh takes
+// several steps in the same grouping and rounding (PAIR_FORM).  Check steps and stored-field steps stay on
+// step_node, which reads and writes the same buffers.
 #pragma once
 
 #include "lbm_kernels.cuh"
@@ -77,20 +79,15 @@ __device__ __forceinline__ float2 p_store(__half *p0, __half *p1, bool has1, flo
     return __half22float2(h);
 }
 
-// Which plain steps run in pairs (chosen per kernel by measurement).  They must be the ones
-// whose single-node steps take the reader-side boundary form.
+// Which plain steps have this grouping: FP16 storage (2-D here, 3-D in lbm_row.cuh).  They must be the
+// ones whose single-node steps take the reader-side boundary form.
 template <int DIM, typename ST> struct PairedStep {
     static constexpr bool value = std::is_same<ST, __half>::value;
     static_assert(!value || ReaderBoundaries<DIM, ST>::step, "paired and single-node steps share one boundary form");
 };
 
-// Resident blocks of 256 threads per SM: 3-D pairs hold 2 x 19 flow populations at once (80
-// registers), 2-D pairs 2 x 9 (48).  Measured on the 256x128x128 electrode and the 4096x1024
-// anode: 3-D 117.5 us at 3 blocks against 121.1 at 4 and 141.8 at 2; 2-D 58.7 us at 5 blocks
-// against 62.6 at 4.
-template <int DIM, typename ST> struct PairOccupancy {
-    static constexpr int blocks = DIM == 3 ? 3 : 5;
-};
+// Resident blocks of 256 threads per SM (48 registers; 4096x1024 anode: 58.7 us at 5 blocks, 62.6 at 4).
+enum : int { PAIR_BLOCKS = 5 };
 
 // The link words of nodes (x, y, z) and (x, y + 1, z) (the second repeats the first where y + 1 =
 // ny), and the element offset of the first.
@@ -269,22 +266,21 @@ __device__ __forceinline__ void step_pair(const StepArgs<DIM, ST> &a, int x0, in
     }
 }
 
-// Plain coupled step, two rows per thread: grid (row / block, ceil(ny / 2), nz).  Both
-// dimensions take the reader-side boundary form (tiles that touch no open boundary run code with
-// no boundary handling): 3-D 109.9 against 117.6 us in the writer form.  The single-node steps
-// of the same storage type take it too (ReaderBoundaries), so that the forms never mix on one
-// lattice.
+// Plain coupled step, two rows per thread: grid (row / block, ceil(ny / 2)), in the reader-side
+// boundary form (tiles that touch no open boundary run code with no boundary handling).  The
+// single-node steps of the same storage type take it too (ReaderBoundaries), so that the forms
+// never mix on one lattice.
 // (A loop over several row pairs per thread, loading the next pair's link words ahead, measured
 // slower at every depth tried.)
 template <int DIM, typename ST, int SINK>
-__global__ void __launch_bounds__(256, PairOccupancy<DIM, ST>::blocks) lbm_pair_kernel(const StepArgs<DIM, ST> a)
+__global__ void __launch_bounds__(256, PAIR_BLOCKS) lbm_pair_kernel(const StepArgs<DIM, ST> a)
 {
     const int x0 = blockIdx.x * blockDim.x;
     const int x = x0 + (int)threadIdx.x;
     if (x >= a.geo.nx) return;
     const int y = 2 * (int)blockIdx.y;
-    // 3-D: the last plane first, as in lbm_step_kernel
-    const int z = DIM == 3 ? (blockIdx.z == 0 ? (int)gridDim.z - 1 : (int)blockIdx.z - 1) : 0;
+    static_assert(DIM == 2, "3-D plain steps are lbm_row.cuh's");
+    const int z = 0;
     uint32_t L[2];
     pair_links(a, x, y, z, L);
     const int y1 = y + 1 < a.geo.ny ? y + 1 : y;
