@@ -10,11 +10,12 @@
 //   - A block loses one row at either edge, a warp two columns at either end; a column's first and last planes
 //     are stepped once more by its neighbours.
 // Bound by latency at 8 warps of 252 registers per SM (no spills): 39% of issue slots used, 880 MB of DRAM traffic
-// per two 256x128x128 steps at 3.4 TB/s; a turn of a plane takes 2.6 us, a third of it for the edges.  The rows are what the registers allow (12 rows at 168
-// registers: 168 us per 256x128x128 step instead of 134, rings of planes in shared memory instead of registers
-// 156 to 170).  us per step, one step per launch and two: 120x120x120 57.4 and 53.3, 256x128x128 135.7 and
-// 134.3, 256x256x128 268 and 250, 300x200x150 307 and 248.  The rule for which lattices is march_shape's.
-// (Flow or transport alone, and FP16 storage, are faster in the row kernel at every size.)
+// per two 256x128x128 steps at 3.4 TB/s; a turn of a plane takes 2.6 us, a third of it for the edges.  The rows
+// are what the registers allow (12 rows at 168 registers: 168 us per 256x128x128 step instead of 134; rings of
+// planes in shared memory instead of registers: 156 to 170).  us per step, one step per launch and two:
+// 120x120x120 57.4 and 53.3, 256x128x128 135.7 and 134.3, 256x256x128 268 and 250, 300x200x150 307 and 248.
+// The rule for which lattices is march_shape's.  (Flow or transport alone, and FP16 storage, are faster in the
+// row kernel at every size.)
 // The rounding is that of the one-step kernels (lbm_collide.cuh): two steps here give the bits of two launches
 // of lbm_row_kernel, and leave the same ghost cells.
 //
