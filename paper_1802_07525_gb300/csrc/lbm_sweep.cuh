@@ -85,9 +85,6 @@ template <int AQ, bool FLOW, bool ADE> struct SweepStage {
     uint2 L;       // links of the row
     bool links;    // any in the warp (uniform)
     float2 uf[2];  // frozen velocity (transport without flow)
-    // the row's inlet value of the one flow direction going down and inwards (formed with the row: the
-    // same sum taken when the row above arrives came out of nvcc 13.0 with that row's population)
-    float in_down;
 };
 
 // Gather the populations along c_i with c_iy < 0 (DOWN: from the row above, `above`) or >= 0 (from
@@ -95,8 +92,7 @@ template <int AQ, bool FLOW, bool ADE> struct SweepStage {
 template <typename ST, int AQ, int SINK, int Q, bool FLOWSET, bool DOWN, bool EDGE, typename D, typename FB, typename FO,
           typename FA>
 __device__ __forceinline__ void sweep_gather(const StepArgs<2, ST, AQ> &a, D &d, const FB &below, const FO &own,
-                                             const FA &above, uint2 L, bool links, const SweepEdge &edge,
-                                             float in_down = 0.0f)
+                                             const FA &above, uint2 L, bool links, const SweepEdge &edge)
 {
     using F = FlowSet<2>;  // the transport sets are its first directions
     const ST *tag = nullptr;
@@ -114,7 +110,6 @@ __device__ __forceinline__ void sweep_gather(const StepArgs<2, ST, AQ> &a, D &d,
         }
         if (EDGE && cx == 1 && edge.inlet) {  // moving-wall bounce-back, or the transport inlet value
             if constexpr (!FLOWSET) d[i].x = ghost_value<AQ, SINK>(tag, a.gin_dev[i < AQ ? i : 0]);
-            else if constexpr (DOWN) d[i].x = in_down;
             else d[i].x = ghost_value<AQ, SINK>(tag, own(F::opp(i)).x + a.bb_in[i]);
         }
     }
@@ -144,8 +139,7 @@ __device__ __forceinline__ void sweep_arrive(const StepArgs<2, ST, AQ> &a, Sweep
 #pragma unroll
         for (int i = 0; i < 9; ++i)
             if (F::c(i, 1) >= 0) out.f[i] = st.got.f[i];
-        sweep_gather<ST, AQ, SINK, 9, true, true, EDGE>(a, out.f, none, held, now, st.L, st.links, edge, st.in_down);
-        if (EDGE) st.in_down = ghost_value<AQ, SINK>((const ST *)nullptr, v.f[6].x + a.bb_in[8]);
+        sweep_gather<ST, AQ, SINK, 9, true, true, EDGE>(a, out.f, none, held, now, st.L, st.links, edge);
         st.got.f[0] = v.f[0];
         sweep_gather<ST, AQ, SINK, 9, true, false, EDGE>(a, st.got.f, held, now, none, L, links, edge);
 #pragma unroll
@@ -319,12 +313,18 @@ __device__ __forceinline__ void sweep_strip(const StepArgs<2, ST, AQ> &a, int x0
 
     // turn q: raw row q arrives at stage 1, which steps row q - 1, which arrives at stage 2, ...; stage
     // T steps row q - T, which is written.  Row q + 1 is loaded as soon as row q has been gathered from.
+    // The stages start from zeros, although what the first turns gather from them is dropped: from an
+    // indeterminate start the compiler may take a held value for the arriving one in every turn (it did,
+    // for the inlet value of the direction going down).
     SweepStage<AQ, FLOW, ADE> st[T];
 #pragma unroll
     for (int s = 0; s < T; ++s) {
+#pragma unroll
+        for (int i = 0; i < (FLOW ? 9 : 0); ++i) st[s].got.f[i] = st[s].up.f[i] = p_all(0.0f);
+#pragma unroll
+        for (int i = 0; i < (ADE ? AQ : 0); ++i) st[s].got.g[i] = st[s].up.g[i] = p_all(0.0f);
         st[s].L = make_uint2(0, 0);
         st[s].links = false;
-        st[s].in_down = 0.0f;
         st[s].uf[0] = st[s].uf[1] = p_all(0.0f);
     }
     Raw in = {};
@@ -504,8 +504,7 @@ __device__ __forceinline__ void tile_steps(const StepArgs<2, ST, AQ> &a, float2 
             auto own = [&](int i) { return v.f[i]; };
             d.f[0] = v.f[0];
             sweep_gather<ST, AQ, SINK, 9, true, false, EDGE>(a, d.f, below, own, above, L, links, edge);
-            sweep_gather<ST, AQ, SINK, 9, true, true, EDGE>(a, d.f, below, own, above, L, links, edge,
-                                                      EDGE ? ghost_value<AQ, SINK>((const ST *)nullptr, v.f[6].x + a.bb_in[8]) : 0.0f);
+            sweep_gather<ST, AQ, SINK, 9, true, true, EDGE>(a, d.f, below, own, above, L, links, edge);
         }
         if constexpr (ADE) {
             auto below = [&](int i) { return below_row[X::place(true, i) * 32]; };
