@@ -462,16 +462,22 @@ def time_plain_steps(P, lat, stream, M=400):
     return graph_ms, e0.elapsed_time(e1) / M
 
 
-def plain_kernel(dim, prec_bytes, nodes, ade_q=0):
-    """The kernel that long runs of plain steps of a bench workload take, and the steps that it carries per
-    launch: in 2-D strips of two (D2Q9 transport: three) from a million nodes on, below that tiles of up to
-    eight; in 3-D two steps per launch in FP32 at the electrode's size, else one."""
+def plain_kernel(lat, prec_bytes, ade_q=0):
+    """The kernel that long runs of a lattice's plain steps take, and the steps that it carries per launch."""
     t = "half" if prec_bytes == 2 else "float"
-    if dim == 2:
-        if nodes > 1000000:
-            return "lbm_sweep_kernel<%s,d2q%d>" % (t, ade_q or 5), 3 if ade_q == 9 else 2
-        return "lbm_tile_kernel<%s>" % t, 8
-    return ("lbm_march_kernel", 2) if prec_bytes == 4 else ("lbm_row_kernel<half>", 1)
+    plan = lat.plain_plan(400)
+    name = {"node": "lbm_step_kernel<%s>" % t, "pair": "lbm_pair_kernel<%s>" % t, "row": "lbm_row_kernel<%s>" % t,
+            "strip": "lbm_sweep_kernel<%s,d2q%d>" % (t, ade_q or 5), "tile": "lbm_tile_kernel<%s>" % t,
+            "march": "lbm_march_kernel"}[plan["kernel"]]
+    return name, plan["steps"]
+
+
+def block_launches(lat, n, block):
+    """Kernel launches of a solve block of n steps: the plain steps', the check step and its sums (two kernels
+    from 2049 partial sums on, one per block of nodes along a row)."""
+    nx, rest = lat.shape[0], math.prod(lat.shape[1:])
+    plain = lat.plain_plan(n - 1)["launches"] if n > 1 else 0
+    return plain + 1 + (2 if -(-nx // block) * rest > 2048 else 1)
 
 
 def step_bytes(dim, prec_bytes, flow_open, ade_open, ade_q=0):
@@ -522,7 +528,7 @@ def leg_variants(P, peak):
         lat.set_launch(block=lat.get_launch()["block"], offsets32=1)
         sb = 2 if prec == P.MFC_FP16_DEV else 4
         byt = step_bytes(w.dim, sb, fo, ao, aq)
-        kname, spl = plain_kernel(w.dim, sb, w.nodes, aq)
+        kname, spl = plain_kernel(lat, sb, aq)
         ach = byt / (spl * kern_ms * 1e-3) / 1e9
         out[name] = {"mlups": w.nodes * steps / (ms * 1e-3) / 1e6, "steps": steps,
                      "kernel_ms": kern_ms, "kernel_ms_direct": kern_direct_ms,
@@ -871,7 +877,9 @@ def main():
     working_set = 2 * sb * (qf + qa) * w.nodes
     bytes_per_launch = step_bytes(w.dim, sb, flow_open, ade_open)
     peak, peak_kind = measured_peaks()
-    kname, spl = plain_kernel(w.dim, sb, w.nodes)
+    kname, spl = plain_kernel(lat, sb)
+    block = lat.get_launch()["block"]
+    gpu_launches = sum(block_launches(lat, min(K, args.steps - s), block) for s in range(0, args.steps, K))
     # a launch of several steps reads and writes every population once
     achieved = bytes_per_launch / (spl * kern_ms * 1e-3) / 1e9
     traffic = traffic_record(kname)
@@ -936,10 +944,6 @@ def main():
         cpu = cpu_baseline(w)
 
     if rank == 0:
-        nblocks = (args.steps + K - 1) // K
-        # per block: the plain steps' launches, the check step and the sums (two kernels from 2048
-        # partials on, one per 256 nodes)
-        launches = nblocks * ((K - 1 + spl - 1) // spl + 1 + (2 if w.nodes > 2048 * 256 else 1))
         line = {
             "metric": METRIC, "value": value, "unit": "MLUPS", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms / args.steps,
@@ -969,7 +973,7 @@ def main():
                     "updates_per_step": args.e2e_steps, "check_every": K_e2e,
                     "path": "mfc_set_geometry (pinned host classes) + mfc_solve_steady + "
                             "mfc_read_fields (rho, u, C, current into pinned host buffers)"},
-            "gpu_launches": launches,
+            "gpu_launches": gpu_launches,
             "clocks": clocks.summary(),
             "final": {"res_flow": res.res_flow, "res_ade": res.res_ade, "current": res.current},
         }

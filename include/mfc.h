@@ -352,6 +352,15 @@ typedef struct {
 MFC_API mfc_status mfc_set_launch(mfc_lattice *lat, const mfc_launch *launch);
 MFC_API mfc_status mfc_get_launch(mfc_lattice *lat, mfc_launch *launch);
 
+/* Kernels of plain steps: one step with one node, two rows' nodes or two nodes of a row per thread; several
+ * steps in strips or tiles (2-D) or along columns of planes (3-D). */
+enum { MFC_KERNEL_NODE = 0, MFC_KERNEL_PAIR = 1, MFC_KERNEL_ROW = 2, MFC_KERNEL_STRIP = 3, MFC_KERNEL_TILE = 4,
+       MFC_KERNEL_MARCH = 5 };
+
+/* How nsteps >= 1 plain steps of `kind` (0 coupled, 1 flow, 2 transport) would be launched: the kernel and the
+ * steps of the first launch (that of the bulk of a long run), and the number of launches.  Outputs may be NULL. */
+MFC_API mfc_status mfc_plain_plan(mfc_lattice *lat, int kind, int nsteps, int *kernel, int *steps, int *launches);
+
 /* ---- slab decomposition (one lattice split along the flow axis) ------------------------- */
 
 /* A lattice too large for one GPU splits along the flow axis into slabs, one per GPU, each a

@@ -34,10 +34,9 @@ cudaError_t launch_sink(const Args &a, const StepHost &h, cudaStream_t s)
     const dim3 grid((unsigned)h.grid, (unsigned)h.geo.ny, (unsigned)h.geo.nz);
     switch (h.mode) {
     case MODE_PLAIN:
-        // one plain step: 32-bit element offsets where the arrays allow them, and two nodes per thread
-        // where that was measured faster (3-D: along a row; 2-D coupled steps in FP16: in two rows)
+        // one plain step: 32-bit element offsets where the arrays allow them, and the kernel of one_step_kernel
         if constexpr (D == 3 && !std::is_same<ST, double>::value) {
-            if (h.idx32) {
+            if (h.kernel == MFC_KERNEL_ROW) {
                 constexpr int FORM = FLOW && ADE && std::is_same<ST, __half>::value ? PAIR_FORM : SCALAR_FORM;
                 const RowPairs rp = row_pairs(h.geo.nx, h.back);
                 const dim3 pairs((unsigned)(((long long)rp.n * h.geo.ny + ROW_BLOCK - 1) / ROW_BLOCK), (unsigned)h.geo.nz);
@@ -45,7 +44,7 @@ cudaError_t launch_sink(const Args &a, const StepHost &h, cudaStream_t s)
                 break;
             }
         } else if constexpr (FLOW && ADE && AQ == default_aq<D>() && PairedStep<D, ST>::value) {
-            if (h.idx32) {
+            if (h.kernel == MFC_KERNEL_PAIR) {
                 const dim3 pairs((unsigned)h.grid, (unsigned)((h.geo.ny + 1) / 2), (unsigned)h.geo.nz);
                 lbm_pair_kernel<D, ST, SINK><<<pairs, h.block, 0, s>>>(a);
                 break;

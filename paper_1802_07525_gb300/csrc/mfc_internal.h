@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "../../include/mfc.h"
 #include "lbm_kernels.cuh"
 
 namespace mfc {
@@ -24,6 +25,7 @@ struct StepHost {
     int nblocks;      // out: blocks of the launch (one reduction partial each)
     int grid, block;  // grid.x (blocks along a row) and threads per block
     SweepShape sweep; // MODE_SWEEP launches
+    int kernel;       // MODE_PLAIN: MFC_KERNEL_NODE, _PAIR or _ROW (see one_step_kernel)
     int back;         // 3-D plain steps: planes from the last to the first (see RowPairs)
     int idx32;        // every population array has fewer than 2^31 elements: 32-bit offsets
     const void *fsrc;

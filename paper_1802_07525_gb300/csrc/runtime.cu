@@ -265,6 +265,25 @@ long long mfc::lattice_max_elements(const mfc_lattice_desc *d)
     return (long long)(l.qf > l.qa ? l.qf : l.qa) * l.geo.plane;
 }
 
+namespace {
+
+// 32-bit element offsets: the largest one a step forms is below max(Q_flow, Q_transport) planes.
+bool offsets_fit(const mfc_lattice *L)
+{
+    return L->offsets32 && std::max(L->qf, L->qa) * L->geo.plane < (1ll << 31);
+}
+
+// The kernel of a single plain step: two nodes per thread where that was measured faster (3-D: along a row;
+// 2-D coupled steps in FP16: in two rows), with 32-bit offsets.
+int one_step_kernel(const mfc_lattice *L, int kind)
+{
+    if (L->dbl || !offsets_fit(L)) return MFC_KERNEL_NODE;
+    if (L->dim == 3) return MFC_KERNEL_ROW;
+    return L->half && kind == KIND_COUPLED && L->qa == 5 ? MFC_KERNEL_PAIR : MFC_KERNEL_NODE;
+}
+
+}  // namespace
+
 void mfc::fill_step(const mfc_lattice *L, int kind, int mode, StepHost *h)
 {
     memset(h, 0, sizeof *h);
@@ -280,9 +299,8 @@ void mfc::fill_step(const mfc_lattice *L, int kind, int mode, StepHost *h)
     h->block = L->block;
     const int q = kind == KIND_FLOW ? L->qf : kind == KIND_ADE ? L->qa : L->qf + L->qa;
     h->back = 2 * q * L->geo.plane * (L->half ? 2 : 4) > BACK_BYTES && (kind == KIND_ADE ? L->gcur : L->fcur);
-    // the largest element offset a step forms is below max(Q_flow, Q_transport) planes
-    const long long qmax = L->qf > L->qa ? L->qf : L->qa;
-    h->idx32 = L->offsets32 && qmax * L->geo.plane < (1ll << 31) ? 1 : 0;
+    h->idx32 = offsets_fit(L);
+    h->kernel = one_step_kernel(L, kind);
     h->fsrc = L->f[L->fcur];
     h->fdst = L->f[1 - L->fcur];
     h->gsrc = L->g[L->gcur];
@@ -341,11 +359,10 @@ namespace {
 bool can_sweep(const mfc_lattice *L, int kind)
 {
     if (L->dim == 3 && (kind != KIND_COUPLED || L->half)) return false;
-    const long long qmax = L->qf > L->qa ? L->qf : L->qa;
     const int fa = L->dim == 2 ? 0 : 2;
     for (int ax = 0; ax < L->dim; ++ax)
         if (L->desc.bc[ax] == MFC_BC_PERIODIC || (ax != fa && L->desc.bc[ax] != MFC_BC_WALL)) return false;
-    return !L->dbl && L->offsets32 && qmax * L->geo.plane < (1ll << 31) && !L->desc.cut[0] && !L->desc.cut[1];
+    return !L->dbl && offsets_fit(L) && !L->desc.cut[0] && !L->desc.cut[1];
 }
 
 // Column tiles and strips of a 2-D sweep of T steps.  The tiles share the columns evenly (even
@@ -482,8 +499,9 @@ mfc_status enqueue_step(mfc_lattice *L, int kind, int mode, int *nblocks = nullp
     return MFC_OK;
 }
 
-// Queue n plain steps of `kind`, several at a time where they can go so.
-mfc_status enqueue_plain(mfc_lattice *L, int kind, int n)
+// Split n plain steps of `kind` into launches, several steps at a time where they can go so: launch(shape) for
+// each, with a null shape for a single step; it stops at the first status that is not MFC_OK.
+template <typename Launch> mfc_status plan_plain(const mfc_lattice *L, int kind, int n, Launch launch)
 {
     SweepShape s;
     const bool sweep = n >= 2 && can_sweep(L, kind) && (L->dim == 2 || march_shape(L, &s));
@@ -495,15 +513,22 @@ mfc_status enqueue_plain(mfc_lattice *L, int kind, int n)
                 s = next_sweep(L, kind, n);
                 shaped_for = n;
             }
-            st = enqueue_step(L, kind, MODE_SWEEP, nullptr, &s);
+            st = launch(&s);
             n -= s.steps;
         } else {
-            st = enqueue_step(L, kind, MODE_PLAIN);
+            st = launch(nullptr);
             n -= 1;
         }
         if (st != MFC_OK) return st;
     }
     return MFC_OK;
+}
+
+mfc_status enqueue_plain(mfc_lattice *L, int kind, int n)
+{
+    return plan_plain(L, kind, n, [&](const SweepShape *s) {
+        return enqueue_step(L, kind, s ? MODE_SWEEP : MODE_PLAIN, nullptr, s);
+    });
 }
 
 // Rewrite the ghost cells of the current buffers from the state they hold.
@@ -1316,6 +1341,26 @@ MFC_API mfc_status mfc_get_launch(mfc_lattice *L, mfc_launch *v)
     if (!L || !v) return MFC_ERR_ARG;
     v->block = L->block;
     v->offsets32 = L->offsets32;
+    return MFC_OK;
+}
+
+MFC_API mfc_status mfc_plain_plan(mfc_lattice *L, int kind, int nsteps, int *kernel, int *steps, int *launches)
+{
+    if (!L) return MFC_ERR_ARG;
+    if (kind < KIND_COUPLED || kind > KIND_ADE || nsteps < 1)
+        return fail(L, MFC_ERR_ARG, "kind must be 0, 1 or 2 and nsteps >= 1");
+    int n = 0, first_kernel = one_step_kernel(L, kind), first_steps = 1;
+    plan_plain(L, kind, nsteps, [&](const SweepShape *s) {
+        if (s && n == 0) {
+            first_kernel = L->dim == 3 ? MFC_KERNEL_MARCH : (s->tile ? MFC_KERNEL_TILE : MFC_KERNEL_STRIP);
+            first_steps = s->steps;
+        }
+        ++n;
+        return MFC_OK;
+    });
+    if (kernel) *kernel = first_kernel;
+    if (steps) *steps = first_steps;
+    if (launches) *launches = n;
     return MFC_OK;
 }
 

@@ -29,6 +29,7 @@ MFC_FP32, MFC_FP16_DEV, MFC_FP64 = 0, 1, 2
 MFC_SEQUENTIAL, MFC_CONCURRENT = 0, 1
 MFC_OUTLET_ZERO_GRADIENT, MFC_OUTLET_DIRICHLET = 0, 1
 MFC_POP_FLOW, MFC_POP_ADE, MFC_FIELD_VELOCITY = 0, 1, 2
+PLAIN_KERNELS = ("node", "pair", "row", "strip", "tile", "march")  # MFC_KERNEL_*
 
 
 class LatticeDesc(ctypes.Structure):
@@ -159,6 +160,7 @@ _SIGS = {
     "mfc_synchronize": (ctypes.c_int, [_vp]),
     "mfc_set_launch": (ctypes.c_int, [_vp, ctypes.POINTER(Launch)]),
     "mfc_get_launch": (ctypes.c_int, [_vp, ctypes.POINTER(Launch)]),
+    "mfc_plain_plan": (ctypes.c_int, [_vp, ctypes.c_int, ctypes.c_int] + [ctypes.POINTER(ctypes.c_int)] * 3),
     "mfc_check_build": (ctypes.c_int, []),
     "mfc_check_canaries": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_longlong)]),
     "mfc_field_sums_noalloc": (ctypes.c_int, [ctypes.c_longlong, ctypes.c_int, _vp, _vp, _vp, _vp,
@@ -415,6 +417,13 @@ class Lattice:
         v = Launch()
         self._check(self._L.mfc_get_launch(self.handle, ctypes.byref(v)))
         return v.as_dict()
+
+    def plain_plan(self, nsteps, kind=0) -> dict:
+        """How nsteps plain steps of kind (0 coupled, 1 flow, 2 transport) are launched: the kernel (node, pair,
+        row, strip, tile or march) and steps of the first launch, and the number of launches."""
+        v = [ctypes.c_int() for _ in range(3)]
+        self._check(self._L.mfc_plain_plan(self.handle, int(kind), int(nsteps), *[ctypes.byref(x) for x in v]))
+        return {"kernel": PLAIN_KERNELS[v[0].value], "steps": v[1].value, "launches": v[2].value}
 
     def check_canaries(self) -> int:
         """Guard bytes found changed (checking builds; 0 in other builds)."""
