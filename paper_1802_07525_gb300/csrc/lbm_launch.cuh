@@ -40,7 +40,9 @@ cudaError_t launch_sink(const Args &a, const StepHost &h, cudaStream_t s)
                 constexpr int FORM = FLOW && ADE && std::is_same<ST, __half>::value ? PAIR_FORM : SCALAR_FORM;
                 const RowPairs rp = row_pairs(h.geo.nx, h.back);
                 const dim3 pairs((unsigned)(((long long)rp.n * h.geo.ny + ROW_BLOCK - 1) / ROW_BLOCK), (unsigned)h.geo.nz);
-                lbm_row_kernel<ST, FLOW, ADE, SINK, FORM><<<pairs, ROW_BLOCK, 0, s>>>(a, rp);
+                const bool periodic = h.bc[0] == BC_PERIODIC || h.bc[1] == BC_PERIODIC || h.bc[2] == BC_PERIODIC;
+                if (periodic) lbm_row_kernel<ST, FLOW, ADE, SINK, FORM, true><<<pairs, ROW_BLOCK, 0, s>>>(a, rp);
+                else lbm_row_kernel<ST, FLOW, ADE, SINK, FORM, false><<<pairs, ROW_BLOCK, 0, s>>>(a, rp);
                 break;
             }
         } else if constexpr (FLOW && ADE && AQ == default_aq<D>() && PairedStep<D, ST>::value) {

@@ -215,9 +215,9 @@ __global__ void __launch_bounds__(MARCH_ROWS * 32, 1) lbm_march_kernel(const Ste
                 row_store<7>(a, a.gdst, d.g, k, both);
                 if (inout && (r == 0 || r == nz - 1)) {
                     if (!(Lq.x & (1u << LK::FLOW_SELF)))
-                        row_flow_ends<float, UU, true>(a, x, y, r, k, Lq.x, [&](int i) { return d.f[i].x; }, u2[0].x, u2[1].x, u2[2].x);
+                        row_flow_ends<float, UU, true, false>(a, x, y, r, k, Lq.x, [&](int i) { return d.f[i].x; }, u2[0].x, u2[1].x, u2[2].x);
                     if (both && !(Lq.y & (1u << LK::FLOW_SELF)))
-                        row_flow_ends<float, UU, true>(a, x + 1, y, r, k + 1, Lq.y, [&](int i) { return d.f[i].y; }, u2[0].y, u2[1].y, u2[2].y);
+                        row_flow_ends<float, UU, true, false>(a, x + 1, y, r, k + 1, Lq.y, [&](int i) { return d.f[i].y; }, u2[0].y, u2[1].y, u2[2].y);
                     if (!(Lq.x & (1u << LK::ADE_SELF))) row_ade_ends<float, true>(a, r, k, Lq.x, d.g[6].x);
                     if (both && !(Lq.y & (1u << LK::ADE_SELF))) row_ade_ends<float, true>(a, r, k + 1, Lq.y, d.g[6].y);
                 }

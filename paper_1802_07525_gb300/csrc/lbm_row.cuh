@@ -102,10 +102,67 @@ __device__ __forceinline__ void row_store(const StepArgs<3, ST> &a, ST *dst, con
     }
 }
 
+// The sides of the lattice that a node lies on, and what a population that leaves across one of them meets.
+// On a periodic axis the neighbour that receives it pulls it through the ghost cell one lattice length away
+// (its image: at most one per direction, shifted along every axis that the direction leaves by); other sides
+// have no image.
+struct RowSides {
+    uint32_t at, shut;  // bit 2 axis + (0: low, 1: high): the node is on that side; the side is not periodic
+    int nx, ny, nz;     // shifts along the axes in elements
+};
+template <typename ST> __device__ __forceinline__ RowSides row_sides(const StepArgs<3, ST> &a, int x, int y, int z)
+{
+    const Geo &g = a.geo;
+    RowSides s;
+    s.at = (x == 0 ? 1u : 0u) | (x == g.nx - 1 ? 2u : 0u) | (y == 0 ? 4u : 0u) | (y == g.ny - 1 ? 8u : 0u) |
+           (z == 0 ? 16u : 0u) | (z == g.nz - 1 ? 32u : 0u);
+    s.shut = (a.bc[0] == BC_PERIODIC ? 0u : 3u) | (a.bc[1] == BC_PERIODIC ? 0u : 12u) | (a.bc[2] == BC_PERIODIC ? 0u : 48u);
+    s.nx = g.nx;
+    s.ny = g.ny * g.px;
+    s.nz = g.nz * (int)g.zs;
+    return s;
+}
+// the sides that direction i leaves by, as in RowSides::at
+__host__ __device__ constexpr uint32_t row_exits(int i)
+{
+    uint32_t m = 0;
+    for (int ax = 0; ax < 3; ++ax) {
+        if (FlowSet<3>::c(i, ax) < 0) m |= 1u << (2 * ax);
+        if (FlowSet<3>::c(i, ax) > 0) m |= 2u << (2 * ax);
+    }
+    return m;
+}
+// Offset from a node to the cell through which its population i is pulled next: out is those of the
+// direction's exits that the node is on.
+__device__ __forceinline__ int row_shift(const RowSides &s, int i, uint32_t out)
+{
+    using F = FlowSet<3>;  // the transport set is its first directions
+    int o = 0;
+    if (F::c(i, 0) != 0 && (out & 3u)) o -= F::c(i, 0) * s.nx;
+    if (F::c(i, 1) != 0 && (out & 12u)) o -= F::c(i, 1) * s.ny;
+    if (F::c(i, 2) != 0 && (out & 48u)) o -= F::c(i, 2) * s.nz;
+    return o;
+}
+
+// Ghost cells of one set's written populations across periodic axes, from the node's post-collision populations
+// v in registers.  (Written back from memory by the general loops of ghost_images, and asked for at every node
+// by a call, they cost more than the step: us per step of 128x128x128, before and now, periodic along y 105.5 and
+// 71.9 in FP32, 87.0 and 57.4 in FP16, along x and y 281 and 74.4, 230 and 57.5; between walls 67.2 and 51.7.)
+template <int Q, typename ST, typename V>
+__device__ __forceinline__ void row_images(const StepArgs<3, ST> &a, ST *pop, const RowSides &s, int k, const V &v)
+{
+    const int P = (int)a.geo.plane;
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+        const uint32_t out = row_exits(i) & s.at;
+        if (out && !(out & s.shut)) st(pop + MFC_IDX(i * P + k + row_shift(s, i, out), Q * P), v(i));
+    }
+}
+
 // Ghost cells of the written flow populations that belong to node (x, y, z) at the inlet or the outlet, from
 // its post-collision populations v and velocity in registers: reading them back after the store costs a
 // round trip to L2 per value, which a small lattice's step waits for.
-template <typename ST, typename FORMS, bool WRITER, typename V>
+template <typename ST, typename FORMS, bool WRITER, bool PERIODIC, typename V>
 __device__ __forceinline__ void row_flow_ends(const StepArgs<3, ST> &a, int x, int y, int z, int k, uint32_t L, const V &v,
                                               float u0, float u1, float u2)
 {
@@ -122,9 +179,16 @@ __device__ __forceinline__ void row_flow_ends(const StepArgs<3, ST> &a, int x, i
 #pragma unroll
         for (int i = 1; i < F::Q; ++i) {
             if (F::c(i, 2) != -1) continue;
-            const int rx = x + F::c(i, 0), ry = y + F::c(i, 1);
-            if (rx >= 0 && rx < g.nx && ry >= 0 && ry < g.ny)
-                st(a.fdst + MFC_IDX(i * P + k + zs, F::Q * P), outlet_value<3, FORMS>(i, a.rho_out, u0, u1, u2));
+            if constexpr (PERIODIC) {
+                const RowSides s = row_sides(a, x, y, z);
+                const uint32_t out = row_exits(i) & s.at & 15u;  // the layer beyond the outlet has the node's sides of x and y
+                if (!(out & s.shut))
+                    st(a.fdst + MFC_IDX(i * P + k + zs + row_shift(s, i, out), F::Q * P), outlet_value<3, FORMS>(i, a.rho_out, u0, u1, u2));
+            } else {
+                const int rx = x + F::c(i, 0), ry = y + F::c(i, 1);
+                if (rx >= 0 && rx < g.nx && ry >= 0 && ry < g.ny)
+                    st(a.fdst + MFC_IDX(i * P + k + zs, F::Q * P), outlet_value<3, FORMS>(i, a.rho_out, u0, u1, u2));
+            }
         }
     }
 }
@@ -139,27 +203,6 @@ __device__ __forceinline__ void row_ade_ends(const StepArgs<3, ST> &a, int z, in
     if (z == a.geo.nz - 1 && !a.cut[1]) st(a.gdst + MFC_IDX(6 * P + k + zs, 7 * P), a.ade_dirichlet ? a.gout_dev[6] : v6);
 }
 
-// Lattices with a periodic axis: the periodic images of node (x, y, z), and the images of the outlet values,
-// read back from the node's stored populations.  SET: the velocity set, Q planes at pop.
-template <typename SET, typename ST, typename FORMS, bool FLOWSET, bool WRITER>
-__device__ __noinline__ void row_images(const StepArgs<3, ST> &a, ST *pop, int x, int y, int z, int k, float u0, float u1,
-                                        float u2)
-{
-    const Geo &g = a.geo;
-    const bool images = on_periodic_boundary<3>(g, a.bc, x, y, z);
-    const bool outlet = a.bc[2] == BC_INOUT && z == g.nz - 1 && !a.cut[1] && (FLOWSET || WRITER);
-#pragma unroll
-    for (int i = 1; i < SET::Q; ++i) {
-        if (images) ghost_images<3, SET, ST>(g, a.bc, pop, i, x, y, z, false, ldplain(pop + (long long)i * g.plane + k));
-        if (outlet && SET::c(i, 2) == -1) {
-            float v;
-            if constexpr (FLOWSET) v = outlet_value<3, FORMS>(i, a.rho_out, u0, u1, u2);
-            else v = a.ade_dirichlet ? a.gout_dev[i] : ldplain(pop + (long long)i * g.plane + k);
-            ghost_images<3, SET, ST>(g, a.bc, pop, i, x, y, g.nz, true, v);
-        }
-    }
-}
-
 // Pairs per row and the multiplier ceil(2^32 / n) of the division by it: the quotient's estimate is at
 // most one too large (q < 2^31), and never too small.
 struct RowPairs {
@@ -172,8 +215,9 @@ struct RowPairs {
     int back;
 };
 
-// One plain step of pair q (numbered along the rows) of plane z.
-template <typename ST, bool FLOW, bool ADE, int SINK, int FORM>
+// One plain step of pair q (numbered along the rows) of plane z.  PERIODIC: whether any axis may be periodic
+// (without, the code for images is left out: its registers cost FP16 flow and transport alone 2%).
+template <typename ST, bool FLOW, bool ADE, int SINK, int FORM, bool PERIODIC>
 __device__ __forceinline__ void row_step(const StepArgs<3, ST> &a, const RowPairs &rp, int q, int z)
 {
     using F = FlowSet<3>;
@@ -195,8 +239,9 @@ __device__ __forceinline__ void row_step(const StepArgs<3, ST> &a, const RowPair
     const bool at_out = READER && a.bc[2] == BC_INOUT && z == g.nz - 1 && !a.cut[1];
     // the node's ghost cells: at the ends of an inlet/outlet axis, and on any boundary of a lattice with a
     // periodic axis
-    const bool periodic = a.bc[0] == BC_PERIODIC || a.bc[1] == BC_PERIODIC || a.bc[2] == BC_PERIODIC;
+    const bool periodic = PERIODIC && (a.bc[0] == BC_PERIODIC || a.bc[1] == BC_PERIODIC || a.bc[2] == BC_PERIODIC);
     const bool ends = valid && a.bc[2] == BC_INOUT && (z == 0 || z == g.nz - 1);
+    const bool images = valid && periodic && (x == 0 || x + 2 >= g.nx || y == 0 || y == g.ny - 1 || z == 0 || z == g.nz - 1);
     float2 u[3] = {p_all(0.0f), p_all(0.0f), p_all(0.0f)};
     float2 e[7];
     if constexpr (FLOW) {
@@ -207,12 +252,18 @@ __device__ __forceinline__ void row_step(const StepArgs<3, ST> &a, const RowPair
         if (valid) row_store<F::Q>(a, a.fdst, d, k, both);
         const bool o0 = valid && !(L.x & (1u << LK::FLOW_SELF)), o1 = valid && both && !(L.y & (1u << LK::FLOW_SELF));
         if (ends) {
-            if (o0) row_flow_ends<ST, UU, !READER>(a, x, y, z, k, L.x, [&](int i) { return d[i].x; }, u[0].x, u[1].x, u[2].x);
-            if (o1) row_flow_ends<ST, UU, !READER>(a, x + 1, y, z, k + 1, L.y, [&](int i) { return d[i].y; }, u[0].y, u[1].y, u[2].y);
+            // FP32 flow alone, one node after the other: written out twice, more spills (flow step of 97x71x83 19.4
+            // against 18.5 us); the other kernels are faster written out (FP16 256x128x128 95.1 against 96.6 us)
+            constexpr int NODES = sizeof(ST) == 4 && !ADE ? 1 : 2;
+#pragma unroll NODES
+            for (int n = 0; n < 2; ++n)
+                if (n ? o1 : o0)
+                    row_flow_ends<ST, UU, !READER, PERIODIC>(a, x + n, y, z, k + n, n ? L.y : L.x, [&](int i) { return n ? d[i].y : d[i].x; },
+                                                             n ? u[0].y : u[0].x, n ? u[1].y : u[1].x, n ? u[2].y : u[2].x);
         }
-        if (periodic) {
-            if (o0) row_images<F, ST, UU, true, !READER>(a, a.fdst, x, y, z, k, u[0].x, u[1].x, u[2].x);
-            if (o1) row_images<F, ST, UU, true, !READER>(a, a.fdst, x + 1, y, z, k + 1, u[0].y, u[1].y, u[2].y);
+        if (images) {
+            if (o0) row_images<F::Q>(a, a.fdst, row_sides(a, x, y, z), k, [&](int i) { return d[i].x; });
+            if (o1) row_images<F::Q>(a, a.fdst, row_sides(a, x + 1, y, z), k + 1, [&](int i) { return d[i].y; });
         }
     }
     if constexpr (ADE) {
@@ -236,22 +287,22 @@ __device__ __forceinline__ void row_step(const StepArgs<3, ST> &a, const RowPair
             if (o0) row_ade_ends<ST, !READER>(a, z, k, L.x, e[6].x);
             if (o1) row_ade_ends<ST, !READER>(a, z, k + 1, L.y, e[6].y);
         }
-        if (periodic) {
-            if (o0) row_images<AdeSet<3>, ST, UU, false, !READER>(a, a.gdst, x, y, z, k, 0.0f, 0.0f, 0.0f);
-            if (o1) row_images<AdeSet<3>, ST, UU, false, !READER>(a, a.gdst, x + 1, y, z, k + 1, 0.0f, 0.0f, 0.0f);
+        if (images) {
+            if (o0) row_images<7>(a, a.gdst, row_sides(a, x, y, z), k, [&](int i) { return e[i].x; });
+            if (o1) row_images<7>(a, a.gdst, row_sides(a, x + 1, y, z), k + 1, [&](int i) { return e[i].y; });
         }
     }
 }
 
 // One plain step of a lattice: grid (pairs of a plane / block, nz); the outlet plane first, whose ghost work is
 // longest.
-template <typename ST, bool FLOW, bool ADE, int SINK, int FORM>
+template <typename ST, bool FLOW, bool ADE, int SINK, int FORM, bool PERIODIC>
 __global__ void __launch_bounds__(ROW_BLOCK, RowOccupancy<ST, FLOW && ADE>::blocks)
     lbm_row_kernel(const StepArgs<3, ST> a, const RowPairs rp)
 {
     const int z = rp.back ? (int)(gridDim.y - 1 - blockIdx.y) : blockIdx.y == 0 ? (int)gridDim.y - 1 : (int)blockIdx.y - 1;
     const int b = (int)(rp.back ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
-    row_step<ST, FLOW, ADE, SINK, FORM>(a, rp, b * ROW_BLOCK + (int)threadIdx.x, z);
+    row_step<ST, FLOW, ADE, SINK, FORM, PERIODIC>(a, rp, b * ROW_BLOCK + (int)threadIdx.x, z);
 }
 
 __host__ __device__ __forceinline__ RowPairs row_pairs(int nx, int back = 0)
@@ -273,6 +324,7 @@ __global__ void __launch_bounds__(ROW_BLOCK, RowOccupancy<ST, true>::blocks) lbm
     const bool back = b.parity && n > (int)(BACK_BYTES / (2 * ROW_BLOCK * 26 * 2 * sizeof(ST)));
     int cur = -1;
     RowPairs rp = {1, 0, 0};
+    bool periodic = false;
     for (int t = blockIdx.x; t < n; t += gridDim.x) {
         const Tile tile = b.tiles[back ? n - 1 - t : t];
         if (tile.slot != cur) {  // uniform over the block
@@ -283,8 +335,10 @@ __global__ void __launch_bounds__(ROW_BLOCK, RowOccupancy<ST, true>::blocks) lbm
             __syncthreads();
             cur = tile.slot;
             rp = row_pairs(sa.geo.nx);
+            periodic = sa.bc[0] == BC_PERIODIC || sa.bc[1] == BC_PERIODIC || sa.bc[2] == BC_PERIODIC;
         }
-        row_step<ST, true, true, SINK_RUNTIME, SCALAR_FORM>(sa, rp, tile.x0 + (int)threadIdx.x, tile.z);
+        if (periodic) row_step<ST, true, true, SINK_RUNTIME, SCALAR_FORM, true>(sa, rp, tile.x0 + (int)threadIdx.x, tile.z);
+        else row_step<ST, true, true, SINK_RUNTIME, SCALAR_FORM, false>(sa, rp, tile.x0 + (int)threadIdx.x, tile.z);
     }
 }
 
