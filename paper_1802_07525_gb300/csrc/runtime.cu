@@ -396,6 +396,18 @@ void tile_shape(const mfc_lattice *L, int T, int rows, SweepShape *s)
     s->strips = (L->ny + rows - 1) / rows;
 }
 
+// Warps of tile blocks that an SM holds: 65,536 registers over a kernel's, as ptxas allots them (64 a thread for
+// coupled FP32 D2Q5, flow alone and FP32 D2Q9 transport alone, 72 for coupled FP16 or D2Q9 and FP16 D2Q9 transport
+// alone).  Counted as 32 warps, blocks of 16 were taken for two per SM: FP16 2353x100 4.26 us per step, 3.61 now,
+// 1500x150 4.88 and 3.45.  (D2Q5 transport alone, 48 registers, holds 42, but is counted as 32: with 42, 700x700 in
+// the paper's order 7.8 -> 8.7 us, 611x293 3.8 -> 3.6.)
+int tile_warps(const mfc_lattice *L, int kind)
+{
+    if (kind == KIND_FLOW) return 32;
+    if (kind == KIND_ADE) return L->qa == 9 && L->half ? 28 : 32;
+    return L->qa == 5 && !L->half ? 32 : 28;
+}
+
 // Estimated time per step, in us, of a tile launch.  Fitted to launches of 8 to 28 warps and 2 to 8 steps
 // on GB300 (FP32 D2Q9 + D2Q5, 128x64 to 1024x512, within 10%): 1.3 us per launch; per block on an SM 71 ns
 // for each row loaded and 48 ns for each row stepped (in proportion to the populations for the other
@@ -407,7 +419,7 @@ double tile_cost(const mfc_lattice *L, int kind, const SweepShape &s)
     const int T = s.steps, warps = s.rows + 2 * T;
     const double row = planes / 14.0 * (0.048 * T * (s.rows + T - 1) + 0.071 * warps);
     const double blocks = (double)s.ntx * L->ny / s.rows;  // the last strip's rows beyond the lattice are idle
-    const int per_sm = std::max(1, 32 / warps);            // 64 registers
+    const int per_sm = std::max(1, tile_warps(L, kind) / warps);
     const double n = std::max(1.0, ceil(blocks / L->sm_count));
     const double rounds = ceil(n / per_sm);
     const double waits = n <= per_sm ? 1.0 : (per_sm == 1 ? rounds : 0.4 * rounds);
