@@ -408,21 +408,37 @@ int tile_warps(const mfc_lattice *L, int kind)
     return L->qa == 5 && !L->half ? 32 : 28;
 }
 
+// Flat lattices: few rows, which tiles of as many rows span.
+bool flat(const mfc_lattice *L) { return L->ny <= 8; }
+
 // Estimated time per step, in us, of a tile launch.  Fitted to launches of 8 to 28 warps and 2 to 8 steps
 // on GB300 (FP32 D2Q9 + D2Q5, 128x64 to 1024x512, within 10%): 1.3 us per launch; per block on an SM 71 ns
 // for each row loaded and 48 ns for each row stepped (in proportion to the populations for the other
 // sets); 0.37 us of latency per step, paid once for the blocks that run together and mostly hidden where
-// an SM holds two blocks or more.
+// an SM holds two blocks or more.  On flat lattices most blocks have rows beyond the lattice, which neither load nor
+// step nor hide anything: there the rows inside are counted, and every round's latency (on 20 lattices of up to
+// 400000x8 the shapes chosen so are within 1% of the best on average, 10% at most).
 double tile_cost(const mfc_lattice *L, int kind, const SweepShape &s)
 {
     const double planes = (kind == KIND_ADE ? 0 : 9) + (kind == KIND_FLOW ? 0 : L->qa);
     const int T = s.steps, warps = s.rows + 2 * T;
-    const double row = planes / 14.0 * (0.048 * T * (s.rows + T - 1) + 0.071 * warps);
-    const double blocks = (double)s.ntx * L->ny / s.rows;  // the last strip's rows beyond the lattice are idle
+    double loaded = warps, stepped = T * (s.rows + T - 1), hidden = 0.4;
+    double blocks = (double)s.ntx * L->ny / s.rows;  // the last strip's rows beyond the lattice are idle
+    if (flat(L)) {
+        loaded = stepped = 0.0;
+        for (int y0 = 0; y0 < L->ny; y0 += s.rows)
+            for (int t = 0; t <= T; ++t) {
+                const int rows = std::min(L->ny, y0 + s.rows + T - t) - std::max(0, y0 - T + t);
+                (t ? stepped : loaded) += (double)rows / s.strips;
+            }
+        blocks = (double)s.ntx * s.strips;
+        hidden = 1.0;
+    }
+    const double row = planes / 14.0 * (0.048 * stepped + 0.071 * loaded);
     const int per_sm = std::max(1, tile_warps(L, kind) / warps);
     const double n = std::max(1.0, ceil(blocks / L->sm_count));
     const double rounds = ceil(n / per_sm);
-    const double waits = n <= per_sm ? 1.0 : (per_sm == 1 ? rounds : 0.4 * rounds);
+    const double waits = n <= per_sm ? 1.0 : (per_sm == 1 ? rounds : hidden * rounds);
     return (1.3 + 0.37 * T * waits + n * row) / T;
 }
 
@@ -431,7 +447,7 @@ double best_tile(const mfc_lattice *L, int kind, int most, SweepShape *best)
 {
     double least = 1e30;
     for (int T = 2; T <= std::min(most, (int)TILE_STEPS); ++T)
-        for (int rows = 1; rows + 2 * T <= TILE_WARPS; ++rows) {
+        for (int rows = 1; rows + 2 * T <= TILE_WARPS && (!flat(L) || rows <= L->ny); ++rows) {
             SweepShape s;
             tile_shape(L, T, rows, &s);
             const double c = tile_cost(L, kind, s);
@@ -475,7 +491,8 @@ bool march_shape(const mfc_lattice *L, SweepShape *s)
 
 // The shape in which the next of n >= 2 plain steps go.  Strips from a million nodes on, where tiles
 // recompute more than they save (2048x1024 FP32: 23.6 against 25.4 us per step, 4096x1024 FP16: 42 against
-// 47; 1024x512: 7.4 against 7.0 and 8.1 against 7.0).  A long run of steps goes in launches of the
+// 47; 1024x512: 7.4 against 7.0 and 8.1 against 7.0), but not on flat lattices, where strips redo most
+// (400000x3 FP32: 20.6 us per step against 18.5, 200000x8 20.9 against 16.6).  A long run of steps goes in launches of the
 // cheapest tiles, its end in tiles of what is left.
 SweepShape next_sweep(const mfc_lattice *L, int kind, int n)
 {
@@ -484,7 +501,7 @@ SweepShape next_sweep(const mfc_lattice *L, int kind, int n)
         march_shape(L, &s);
         return s;
     }
-    if (L->N > 1000000) {
+    if (L->N > 1000000 && !flat(L)) {
         const int T = L->qa == 9 ? SweepSteps<9>::value : SweepSteps<5>::value;
         sweep_shape(L, T == 3 && (n == 2 || n == 4) ? 2 : std::min(T, n), &s);
         return s;

@@ -48,7 +48,7 @@ def _same(P, a, b):
     ((1203, 853), "MFC_FP32", 0, 0.0, 0), ((1203, 853), "MFC_FP32", 0, 0.05, 1), ((2049, 509), "MFC_FP32", 0, 0.05, 0),
     ((1203, 853), "MFC_FP16_DEV", 0, 0.0, 0), ((509, 2011), "MFC_FP16_DEV", 0, 0.05, 1),
     ((1021, 1013), "MFC_FP32", 9, 0.0, 0), ((2049, 509), "MFC_FP32", 9, 0.05, 1),
-    ((1203, 853), "MFC_FP16_DEV", 9, 0.0, 1), ((17, 65535), "MFC_FP32", 0, 0.0, 0), ((200003, 6), "MFC_FP32", 0, 0.0, 0),
+    ((1203, 853), "MFC_FP16_DEV", 9, 0.0, 1), ((17, 65535), "MFC_FP32", 0, 0.0, 0), ((90001, 12), "MFC_FP32", 0, 0.0, 0),
 ], ids=str)
 def test_strips_compute_what_single_steps_compute(P, shape, prec, ade_q, k_half, outlet):
     a, b = _pair(P, shape, precision=getattr(P, prec), ade_q=ade_q, k_half=k_half, ade_outlet=outlet)

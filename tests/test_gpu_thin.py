@@ -42,3 +42,29 @@ def test_3d_thin_planes_cost_no_more_than_one_node_per_thread(P, prec):
         pairs = _best(g, 60, g.step_coupled_plain)
         g.set_launch(block=128, offsets32=0)
         assert pairs < _best(g, 60, g.step_coupled_plain)
+
+
+FLAT = [(200000, 1), (200001, 2), (110000, 5), (200000, 4), (400001, 3), (60000, 6), (130001, 8), (7, 2), (1, 1)]
+
+
+@pytest.mark.parametrize("shape", FLAT, ids=str)
+@pytest.mark.parametrize("prec,ade_q", [("MFC_FP32", 0), ("MFC_FP16_DEV", 0), ("MFC_FP32", 9)])
+def test_2d_flat_lattices_compute_what_single_steps_compute(P, shape, prec, ade_q):
+    out = []
+    for n in (11, 1):
+        with _lattice(P, shape, precision=getattr(P, prec), ade_q=ade_q) as g:
+            assert g.plain_plan(11)["kernel"] == "tile"
+            for _ in range(11 // n):
+                g.step_coupled_plain(n)
+            out.append([g.read_populations(w) for w in (P.MFC_POP_FLOW, P.MFC_POP_ADE)])
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("shape", [(200000, 1), (200000, 4), (400000, 2), (110000, 5)], ids=str)
+@pytest.mark.parametrize("prec", ["MFC_FP32", "MFC_FP16_DEV"])
+def test_2d_flat_lattices_cost_no_more_than_single_steps(P, shape, prec):
+    """Tiles were chosen as if their rows beyond a lattice cost nothing: up to five times a single step's time."""
+    with _lattice(P, shape, precision=getattr(P, prec)) as g:
+        several = _best(g, 48, g.step_coupled_plain)
+        assert several < _best(g, 48, lambda n: [g.step_coupled_plain(1) for _ in range(n)])
