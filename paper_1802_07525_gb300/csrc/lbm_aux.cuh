@@ -63,40 +63,43 @@ __device__ __forceinline__ void node_xyz(const Geo &g, long long q, int *x, int 
     *z = (int)(q / ((long long)g.nx * g.ny));
 }
 
-// Is the link that brings a population along (cx,cy,cz) to (x,y,z) blocked (Eq. 11)?  Walls win
-// over the inlet and outlet; a periodic source wraps; an outlet source moves back onto the last
-// layer, whose class decides; a source beyond a cut is the neighbouring slab's node, whose class
-// the halo plane gives.
+// The class that decides whether the link that brings a population along (cx,cy,cz) to node q at (x,y,z) is
+// blocked (Eq. 11): its source's, where that is a node.  Beyond the lattice walls win over the inlet and outlet
+// (blocked for both sets); a periodic source wraps; an outlet source moves back onto the last layer, whose class
+// decides; an inlet ghost is open; a source beyond a cut is the neighbouring slab's node, whose class the halo
+// plane gives.
 template <int DIM>
-__device__ __forceinline__ bool mask_blocked(const MaskArgs &m, int x, int y, int z, int cx, int cy,
-                                             int cz, uint8_t bit)
+__host__ __device__ __forceinline__ uint8_t link_class(const MaskArgs &m, long long q, int x, int y, int z, int cx, int cy, int cz)
 {
-    int s[3] = {x - cx, y - cy, z - cz};
-    const int n[3] = {m.geo.nx, m.geo.ny, m.geo.nz};
     constexpr int FA = DIM == 2 ? 0 : 2;
-    const int side = s[FA] < 0 ? 0 : (s[FA] >= n[FA] ? 1 : -1);
-    const bool across_cut = side >= 0 && m.cut[side];
+    const int s[3] = {x - cx, y - cy, z - cz};
+    const int n[3] = {m.geo.nx, m.geo.ny, m.geo.nz};
+    const int c[3] = {cx, cy, cz};
+    long long stride = 1;
+    long long from = q - (cx + (long long)m.geo.nx * (cy + (long long)m.geo.ny * cz));
+    bool inlet = false, cut = false;
+#pragma unroll
     for (int ax = 0; ax < DIM; ++ax) {
-        const bool out = s[ax] < 0 || s[ax] >= n[ax];
-        if (ax == FA && across_cut) continue;
-        if (out && !(m.bc[ax] == BC_PERIODIC || (m.bc[ax] == BC_INOUT && ax == FA))) return true;
-    }
-    for (int ax = 0; ax < DIM; ++ax) {
-        if (s[ax] >= 0 && s[ax] < n[ax]) continue;
-        if (ax == FA && across_cut) continue;
-        if (m.bc[ax] == BC_PERIODIC) {
-            s[ax] = s[ax] < 0 ? s[ax] + n[ax] : s[ax] - n[ax];
-        } else {
-            if (s[ax] < 0) return false;  // inlet ghost
-            s[ax] = n[ax] - 1;            // outlet: the last layer decides
+        if (c[ax] != 0 && (c[ax] > 0 ? s[ax] < 0 : s[ax] >= n[ax])) {
+            const int side = c[ax] > 0 ? 0 : 1;
+            if (ax == FA && m.cut[side]) cut = true;
+            else if (m.bc[ax] == BC_PERIODIC) from += c[ax] * n[ax] * stride;
+            else if (!(m.bc[ax] == BC_INOUT && ax == FA)) return CLS_FLOW | CLS_ADE;
+            else if (side == 0) inlet = true;
+            else from -= stride;
         }
+        stride *= n[ax];
     }
-    if (across_cut) {
-        const uint8_t *h = m.halo_cls[side];
-        const long long cross = DIM == 2 ? (long long)s[1] : s[0] + (long long)m.geo.nx * s[1];
-        return h && (h[cross] & bit) != 0;
+    if (inlet) return 0;
+    if (cut) {
+        const uint8_t *h = m.halo_cls[c[FA] > 0 ? 0 : 1];
+        // across the cut the other axes' sources have wrapped already
+        int t[3] = {s[0], s[1], s[2]};
+        for (int ax = 0; ax < DIM; ++ax)
+            if (ax != FA && m.bc[ax] == BC_PERIODIC) t[ax] = t[ax] < 0 ? t[ax] + n[ax] : (t[ax] >= n[ax] ? t[ax] - n[ax] : t[ax]);
+        return h ? h[DIM == 2 ? (long long)t[1] : t[0] + (long long)m.geo.nx * t[1]] : 0;
     }
-    return (m.cls_new[s[0] + (long long)m.geo.nx * (s[1] + (long long)m.geo.ny * s[2])] & bit) != 0;
+    return m.cls_new[from];
 }
 
 // Link words from the node classes; (re)initialise populations and fields of nodes whose class
@@ -118,22 +121,18 @@ template <int DIM, int AQ = default_aq<DIM>()> __global__ void build_links_kerne
         if (c & CLS_FLOW) L |= 1u << LK::FLOW_SELF;
         if (c & CLS_ADE) L |= 1u << LK::ADE_SELF;
         if (c & CLS_SINK) L |= 1u << LK::SINK;
-        // every link of a blocked node bounces back: its (zero) populations stay where they are
-        if (x > 0 && x < m.geo.nx - 1 && y > 0 && y < m.geo.ny - 1 && (DIM == 2 || (z > 0 && z < m.geo.nz - 1))) {
-            // inside, a link's source is a node: one class byte serves both sets (the general form below,
-            // for every node, took 640 us on 256x128x128; with this 250)
+        // every link of a blocked node bounces back: its (zero) populations stay where they are.  One class byte of
+        // the link's source serves both sets, and warps with all nodes inside look no further (biofilm_grow of
+        // 256x128x128, mostly this kernel: 817 us with two searches per link, 387 now; of 60x60x60, where every warp
+        // has nodes at the sides, 101 and 66, 108 with a node's own choice between the two ways)
+        const bool inside = x > 0 && x < m.geo.nx - 1 && y > 0 && y < m.geo.ny - 1 && (DIM == 2 || (z > 0 && z < m.geo.nz - 1));
+        const bool all_inside = __all_sync(__activemask(), inside);
 #pragma unroll
-            for (int i = 1; i < F::Q; ++i) {
-                const uint8_t o = m.cls_new[q - (F::c(i, 0) + (long long)m.geo.nx * (F::c(i, 1) + (long long)m.geo.ny * F::c(i, 2)))];
-                if ((c | o) & CLS_FLOW) L |= 1u << i;
-                if (i < A::Q && ((c | o) & CLS_ADE)) L |= 1u << (LK::ADE_SELF + i);
-            }
-        } else {
-            for (int i = 1; i < F::Q; ++i)
-                if ((c & CLS_FLOW) || mask_blocked<DIM>(m, x, y, z, F::c(i, 0), F::c(i, 1), F::c(i, 2), CLS_FLOW)) L |= 1u << i;
-            for (int i = 1; i < A::Q; ++i)
-                if ((c & CLS_ADE) || mask_blocked<DIM>(m, x, y, z, A::c(i, 0), A::c(i, 1), A::c(i, 2), CLS_ADE))
-                    L |= 1u << (LK::ADE_SELF + i);
+        for (int i = 1; i < F::Q; ++i) {
+            const long long from = q - (F::c(i, 0) + (long long)m.geo.nx * (F::c(i, 1) + (long long)m.geo.ny * F::c(i, 2)));
+            const uint8_t o = c | (all_inside ? m.cls_new[from] : link_class<DIM>(m, q, x, y, z, F::c(i, 0), F::c(i, 1), F::c(i, 2)));
+            if (o & CLS_FLOW) L |= 1u << i;
+            if (i < A::Q && (o & CLS_ADE)) L |= 1u << (LK::ADE_SELF + i);
         }
         reinterpret_cast<LinkT *>(m.link)[k] = (LinkT)L;
 
