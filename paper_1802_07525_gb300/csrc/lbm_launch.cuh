@@ -72,8 +72,9 @@ cudaError_t launch_sink(const Args &a, const StepHost &h, cudaStream_t s)
                 kernel<<<tiles, 32 * warps, warps * row, s>>>(a, h.sweep);
                 break;
             }
-            if (h.sweep.steps == 2) lbm_sweep_kernel<ST, FLOW, ADE, AQ, SINK, FORM, 2><<<tiles, 32, 0, s>>>(a, h.sweep);
-            else lbm_sweep_kernel<ST, FLOW, ADE, AQ, SINK, FORM, SweepSteps<AQ>::value><<<tiles, 32, 0, s>>>(a, h.sweep);
+            constexpr int most = SweepSteps<AQ, FLOW && ADE>::value;
+            if (h.sweep.steps == most) lbm_sweep_kernel<ST, FLOW, ADE, AQ, SINK, FORM, most><<<tiles, 32, 0, s>>>(a, h.sweep);
+            else lbm_sweep_kernel<ST, FLOW, ADE, AQ, SINK, FORM, 2><<<tiles, 32, 0, s>>>(a, h.sweep);
             break;
         }
         if constexpr (D == 3 && std::is_same<ST, float>::value && FLOW && ADE) {

@@ -391,9 +391,11 @@ __device__ __forceinline__ void sweep_strip(const StepArgs<2, ST, AQ> &a, int x0
 
 // Steps per sweep and resident warps per SM, measured: two steps with 12 warps (164 registers) for
 // D2Q9 + D2Q5 (2048x1024 FP32: 24 us per step; with 13 warps, where it spills, 37; with 10, 28; three
-// steps with 8 warps 26); three steps with 8 warps for D2Q9 transport (1024x512: 10.8 against 11.7 us).
-template <int AQ> struct SweepSteps {
-    static constexpr int value = AQ == 9 ? 3 : 2;
+// steps with 8 warps 26).  D2Q9 transport, 8 warps: two steps coupled (240 registers; 2048x1024 FP32 31.5 us, FP16
+// 36.5; three steps spill 112 bytes: 38.0 and 40.7), three for flow alone and transport alone (2048x1024 in the
+// paper's order 32.2 and 38.0 us; two steps 41.1 and 39.8).
+template <int AQ, bool COUPLED> struct SweepSteps {
+    static constexpr int value = AQ == 9 && !COUPLED ? 3 : 2;
 };
 template <int T, int AQ> struct SweepOccupancy {
     static constexpr int blocks = T == 2 && AQ != 9 ? 12 : 8;

@@ -502,7 +502,7 @@ SweepShape next_sweep(const mfc_lattice *L, int kind, int n)
         return s;
     }
     if (L->N > 1000000 && !flat(L)) {
-        const int T = L->qa == 9 ? SweepSteps<9>::value : SweepSteps<5>::value;
+        const int T = L->qa == 9 && kind != KIND_COUPLED ? SweepSteps<9, false>::value : SweepSteps<9, true>::value;
         sweep_shape(L, T == 3 && (n == 2 || n == 4) ? 2 : std::min(T, n), &s);
         return s;
     }

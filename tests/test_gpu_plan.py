@@ -60,3 +60,11 @@ def test_plan_refuses_bad_arguments(P):
             with pytest.raises(P.MfcError) as e:
                 g.plain_plan(n, kind)
             assert e.value.status == P.MFC_ERR_ARG
+
+
+@pytest.mark.parametrize("ade_q,kind,steps", [(0, 0, 2), (0, 1, 2), (0, 2, 2), (9, 0, 2), (9, 1, 3), (9, 2, 3)])
+def test_steps_of_strips(P, ade_q, kind, steps):
+    """Three steps where the registers hold them: D2Q9 flow alone and transport alone, not coupled (which spills)."""
+    with P.Lattice((1203, 853), ade_q=ade_q) as g:
+        assert g.plain_plan(400, kind)["kernel"] == "strip" and g.plain_plan(400, kind)["steps"] == steps
+        assert [g.plain_plan(n, kind)["launches"] for n in (1, 2, 3, 4, 5)] == ([1, 1, 2, 2, 3] if steps == 2 else [1, 1, 1, 2, 2])
