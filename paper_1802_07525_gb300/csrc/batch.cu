@@ -535,6 +535,10 @@ mfc_status autotune(mfc_batch *B)
     return MFC_OK;
 }
 
+// Blocks of one plain and one check step (check_every 2): the 2-D instances' plain step goes by row segments, as a
+// tile loads 10 rows to write 8 (FP32; four anodes of 1.1 million nodes, 200 steps: 18.4 against 19.0 ms).
+bool by_segments(const mfc_batch *B) { return B->K == 2 && !B->half; }
+
 // The graph of one block for the groups in `mask`.
 mfc_status graph_for(mfc_batch *B, int mask, cudaGraphExec_t *out)
 {
@@ -545,13 +549,16 @@ mfc_status graph_for(mfc_batch *B, int mask, cudaGraphExec_t *out)
     BCK(B, cudaStreamBeginCapture(B->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
     // the plain steps group by group (no group waits for another's results), then the check step of all
-    if (mask & HAS_2D) {
+    if (by_segments(B) && (mask & HAS_2D)) {
+        e = launch_batch(batch_host(B, B->grp[0], MODE_PLAIN, 0), B->stream);
+    } else if (mask & HAS_2D) {
         const std::vector<int> plan = sweep_plan(B, B->K - 1);
         for (size_t j = 0; j < plan.size() && e == cudaSuccess; ++j)
             e = launch_batch(fast_host(B, B->grp[0], plan[j], (int)(j & 1)), B->stream);
     }
     for (int s = 0; s < B->K - 1 && e == cudaSuccess; ++s) {
-        if (mask & HAS_2D_SINGLE) e = launch_batch(rest_host(B, B->grp[0], s & 1), B->stream);
+        if ((mask & HAS_2D_SINGLE) && !(by_segments(B) && (mask & HAS_2D)))
+            e = launch_batch(rest_host(B, B->grp[0], s & 1), B->stream);
         if ((mask & HAS_3D) && e == cudaSuccess) e = launch_batch(fast_host(B, B->grp[1], 1, s & 1), B->stream);
     }
     const bool present[NGROUP] = {(mask & (HAS_2D | HAS_2D_SINGLE)) != 0, (mask & HAS_3D) != 0};
