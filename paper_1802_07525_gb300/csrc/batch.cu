@@ -453,37 +453,58 @@ mfc_status set_block(mfc_batch *B, int block)
     return rebuild_tables(B);
 }
 
-// Pick the block size by timing plain steps of the resident instances, and K (when not given)
-// from the measured step time and check overhead.  The timed steps read buffer A and write
-// buffer B of every instance; the next real step rewrites everything of B that is read later,
-// so tuning changes no result.
-mfc_status autotune(mfc_batch *B)
+// Time of a launch of every group, in s: check steps, or the plain steps that row segments take.
+mfc_status time_segments(mfc_batch *B, int mode, double *t)
 {
-    std::vector<int> cand;
-    if (B->opts.block) cand.push_back(B->opts.block);
-    else cand = {64, 128, 256};
-    double best = 1e30;
-    int best_block = cand[0];
-    for (int blk : cand) {
-        mfc_status st = set_block(B, blk);
-        if (st != MFC_OK) return st;
-        const int reps = 5;
-        for (int r = -2; r < reps; ++r) {
-            if (r == 0) BCK(B, cudaEventRecord(B->t0, B->stream));
-            for (int gi = 0; gi < NGROUP; ++gi)
-                if (B->grp[gi].ntiles) BCK(B, launch_batch(batch_host(B, B->grp[gi], MODE_PLAIN, 0), B->stream));
-        }
-        BCK(B, cudaEventRecord(B->t1, B->stream));
-        BCK(B, cudaEventSynchronize(B->t1));
-        float ms = 0.f;
-        BCK(B, cudaEventElapsedTime(&ms, B->t0, B->t1));
-        const double t = ms * 1e-3 / reps;
-        if (t < best) {
-            best = t;
-            best_block = blk;
+    const int reps = 3;
+    for (int r = -1; r < reps; ++r) {
+        if (r == 0) BCK(B, cudaEventRecord(B->t0, B->stream));
+        for (int gi = 0; gi < NGROUP; ++gi) {
+            const Group &g = B->grp[gi];
+            if (mode == MODE_CHECK && g.ntiles) BCK(B, launch_batch(batch_host(B, g, MODE_CHECK, 0), B->stream));
+            if (mode == MODE_PLAIN && g.nrest) BCK(B, launch_batch(rest_host(B, g, 0), B->stream));
         }
     }
-    if (B->block != best_block) {
+    BCK(B, cudaEventRecord(B->t1, B->stream));
+    BCK(B, cudaEventSynchronize(B->t1));
+    float ms = 0.f;
+    BCK(B, cudaEventElapsedTime(&ms, B->t0, B->t1));
+    *t = ms * 1e-3 / reps;
+    return MFC_OK;
+}
+
+// Pick the block size, when not given, by timing what it shapes: the check steps, and the plain steps of 2-D
+// instances that cannot go several at a time; and K, when not given, from the measured step time and check
+// overhead.  The timed steps read buffer A and write buffer B of every instance, of which the next real step
+// rewrites everything that is read later; timed check steps store fields too, which are put back to rest (every
+// instance is new here), so tuning changes no result.
+mfc_status autotune(mfc_batch *B)
+{
+    double best = 1e30;
+    int best_block = B->opts.block;
+    if (!best_block) {
+        for (int blk : {64, 128, 256}) {
+            mfc_status st = set_block(B, blk);
+            if (st != MFC_OK) return st;
+            double check = 0.0, plain = 0.0;
+            st = time_segments(B, MODE_CHECK, &check);
+            if (st == MFC_OK && B->grp[0].nrest) st = time_segments(B, MODE_PLAIN, &plain);
+            if (st != MFC_OK) return st;
+            const double t = check + ((B->K ? B->K : 200) - 1) * plain;  // per block of steps
+            if (t < best) {
+                best = t;
+                best_block = blk;
+            }
+        }
+        for (auto &sl : B->slots) {
+            if (!sl.L || sl.state != SLOT_ACTIVE) continue;
+            const size_t bytes = (size_t)sl.L->geo.plane * sizeof(float);
+            BCK(B, cudaMemsetAsync(sl.L->fld_rho, 0, bytes, B->stream));
+            BCK(B, cudaMemsetAsync(sl.L->fld_u, 0, sl.L->dim * bytes, B->stream));
+            BCK(B, cudaMemsetAsync(sl.L->fld_c, 0, bytes, B->stream));
+        }
+    }
+    if (B->opts.block || B->block != best_block) {
         mfc_status st = set_block(B, best_block);
         if (st != MFC_OK) return st;
     }

@@ -170,6 +170,17 @@ template <typename S> cudaError_t launch_batch_sweep(const BatchArgs<3, S> &b, c
     return cudaGetLastError();
 }
 
+// One plain step of 2-D instances by row segments (3-D ones all take the row kernel).
+template <typename S> cudaError_t launch_batch_plain(const BatchArgs<2, S> &b, const BatchHost &h, cudaStream_t s)
+{
+    lbm_batch_kernel<2, S, true, true, MODE_PLAIN><<<h.grid, h.block, 0, s>>>(b);
+    return cudaGetLastError();
+}
+template <typename S> cudaError_t launch_batch_plain(const BatchArgs<3, S> &, const BatchHost &, cudaStream_t)
+{
+    return cudaErrorInvalidValue;
+}
+
 // Coupled steps only: a batch advances flow and transport of every instance together.
 cudaError_t MFC_BATCH_FN(const BatchHost &h, cudaStream_t s)
 {
@@ -182,18 +193,17 @@ cudaError_t MFC_BATCH_FN(const BatchHost &h, cudaStream_t s)
     switch (h.mode) {
     case MODE_SWEEP:
         return launch_batch_sweep(b, h, s);
-    case MODE_PLAIN: lbm_batch_kernel<D, ST, true, true, MODE_PLAIN><<<h.grid, h.block, 0, s>>>(b); break;
-    case MODE_WRITE: lbm_batch_kernel<D, ST, true, true, MODE_WRITE><<<h.grid, h.block, 0, s>>>(b); break;
+    case MODE_PLAIN: return launch_batch_plain(b, h, s);
     default: lbm_batch_kernel<D, ST, true, true, MODE_CHECK><<<h.grid, h.block, 0, s>>>(b); break;
     }
     return cudaGetLastError();
 }
 
-// Resident blocks per SM of the plain batch step at `block` threads.
+// Resident blocks per SM of the check step of batches at `block` threads (2-D plain steps have the same).
 int MFC_OCC_FN(int block)
 {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, lbm_batch_kernel<D, ST, true, true, MODE_PLAIN>, block, 0) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, lbm_batch_kernel<D, ST, true, true, MODE_CHECK>, block, 0) !=
         cudaSuccess) {
         cudaGetLastError();
         return 1;

@@ -56,3 +56,26 @@ def test_short_blocks(P, prec, every):
         scale = max(np.abs(u).max(), 1e-3)
         assert np.abs(got["u"] - u).max() <= unit * scale
         assert np.abs(got["c"] - c).max() <= unit * max(np.abs(c).max(), 1e-3)
+
+
+@pytest.mark.parametrize("prec", ["MFC_FP32", "MFC_FP16_DEV"])
+def test_tuned_block_gives_the_results_of_the_given_one(P, prec):
+    """Tuning runs check steps, which store fields: the first check must still compare with the state at rest."""
+    prec = getattr(P, prec)
+    tuned = P.Batch(precision=prec, check_every=4)
+    t = [tuned.submit(s, _classes(s), bc=bc, tol_flow=0.0, tol_ade=0.0, max_steps=4, **_kw(s)) for s, bc in REQUESTS]
+    tuned.run()
+    block = tuned.stats()["block"]
+    got = [tuned.poll(x) for x in t]
+    tuned.close()
+    assert block in (64, 128, 256)
+    want = P.Batch(precision=prec, check_every=4, block=block)
+    t = [want.submit(s, _classes(s), bc=bc, tol_flow=0.0, tol_ade=0.0, max_steps=4, **_kw(s)) for s, bc in REQUESTS]
+    want.run()
+    for a, x in zip(got, t):
+        b = want.poll(x)
+        for k in ("rho", "u", "c"):
+            assert np.array_equal(a[k], b[k])
+        for k in ("res_flow", "res_ade", "mass", "current", "steps_flow"):
+            assert a[k] == b[k], k
+    want.close()
