@@ -45,10 +45,10 @@ cudaError_t launch_sink(const Args &a, const StepHost &h, cudaStream_t s)
                 else lbm_row_kernel<ST, FLOW, ADE, SINK, FORM, false><<<pairs, ROW_BLOCK, 0, s>>>(a, rp);
                 break;
             }
-        } else if constexpr (FLOW && ADE && AQ == default_aq<D>() && PairedStep<D, ST>::value) {
+        } else if constexpr (D == 2 && FLOW && ADE && AQ == default_aq<D>() && PairedStep<D, ST>::value) {
             if (h.kernel == MFC_KERNEL_PAIR) {
-                const dim3 pairs((unsigned)h.grid, (unsigned)((h.geo.ny + 1) / 2), (unsigned)h.geo.nz);
-                lbm_pair_kernel<D, ST, SINK><<<pairs, h.block, 0, s>>>(a);
+                const dim3 pairs((unsigned)h.grid, (unsigned)((h.geo.ny + 1) / 2));
+                lbm_pair_kernel<ST, SINK><<<pairs, h.block, 0, s>>>(a);
                 break;
             }
         } else if (h.idx32) {

@@ -65,12 +65,6 @@ __device__ __forceinline__ float2 p_cdot(int i, const float2 (&u)[3], float &s)
 }
 
 // Store the two lanes (lane 1 only where it exists); returns the values the stores keep.
-__device__ __forceinline__ float2 p_store(float *p0, float *p1, bool has1, float2 v)
-{
-    *p0 = v.x;
-    if (has1) *p1 = v.y;
-    return v;
-}
 __device__ __forceinline__ float2 p_store(__half *p0, __half *p1, bool has1, float2 v)
 {
     const __half2 h = __float22half2_rn(v);
@@ -89,52 +83,39 @@ template <int DIM, typename ST> struct PairedStep {
 // Resident blocks of 256 threads per SM (48 registers; 4096x1024 anode: 58.7 us at 5 blocks, 62.6 at 4).
 enum : int { PAIR_BLOCKS = 5 };
 
-// The link words of nodes (x, y, z) and (x, y + 1, z) (the second repeats the first where y + 1 =
-// ny), and the element offset of the first.
-template <int DIM, typename ST>
-__device__ __forceinline__ int pair_links(const StepArgs<DIM, ST> &a, int x, int y, int z, uint32_t (&L)[2])
+// The link words of nodes (x, y) and (x, y + 1) (the second repeats the first where y + 1 = ny).
+template <typename ST>
+__device__ __forceinline__ void pair_links(const StepArgs<2, ST> &a, int x, int y, uint32_t (&L)[2])
 {
     const Geo &g = a.geo;
-    const int k0 = (int)g.row0 + z * (int)g.zs + y * g.px + x;
+    const int k0 = (int)g.row0 + y * g.px + x;
     const int k1 = y + 1 < g.ny ? k0 + g.px : k0;
     L[0] = __ldg(a.link + MFC_IDX(k0, g.plane));
     L[1] = __ldg(a.link + MFC_IDX(k1, g.plane));
-    return k0;
 }
 
-// One plain coupled step of nodes (x0 + threadIdx.x, y + l, z), l = 0, 1 (lane 1 absent where
-// y + 1 = ny; x < nx), given their link words, with 32-bit element offsets and the default
-// transport set.  BFORM as in step_node.
-template <int DIM, typename ST, int BFORM, int SINK>
-__device__ __forceinline__ void step_pair(const StepArgs<DIM, ST> &a, int x0, int y, int z, const uint32_t (&L)[2])
+// One plain coupled step of nodes (x, y + l), l = 0, 1 (lane 1 absent where y + 1 = ny; x < nx), given
+// their link words, with 32-bit element offsets and the default transport set, in the reader form of the
+// open boundaries.  BOUNDARY: the block's tile touches one.
+template <typename ST, bool BOUNDARY, int SINK>
+__device__ __forceinline__ void step_pair(const StepArgs<2, ST> &a, int x, int y, const uint32_t (&L)[2])
 {
-    using F = FlowSet<DIM>;
-    using A = AdeSet<DIM>;
-    using LK = Links<DIM>;
+    using F = FlowSet<2>;
+    using A = AdeSet<2>;
+    using LK = Links<2>;
     static_assert(std::is_same<ArithT<ST>, float>::value, "paired FP32 arithmetic");
     static_assert(!A::quadratic, "linear transport equilibrium");
     const Geo g = a.geo;
-    const int x = x0 + threadIdx.x;
     const bool has1 = y + 1 < g.ny;
     const int P = (int)g.plane;
-    const int k0 = (int)g.row0 + z * (int)g.zs + y * g.px + x;
+    const int k0 = (int)g.row0 + y * g.px + x;
     const int k[2] = {k0, has1 ? k0 + g.px : k0};
-    constexpr bool READER = BFORM != B_WRITER;
-    const int y1 = has1 ? y + 1 : y;
-    const bool bnd_tile = BFORM == B_WRITER ? (tile_on_open_boundary<DIM>(g, a.bc, x0, blockDim.x, y, z) ||
-                                               tile_on_open_boundary<DIM>(g, a.bc, x0, blockDim.x, y1, z))
-                                            : BFORM == B_BOUNDARY;
     bool ghosts[2];
 #pragma unroll
-    for (int l = 0; l < 2; ++l)
-        ghosts[l] = bnd_tile && (l == 0 || has1) &&
-                    (READER ? step_writes_ghosts<DIM>(g, a.bc, x, y + l, z) : on_open_boundary<DIM>(g, a.bc, x, y + l, z));
-    constexpr int FA = flow_axis<DIM>();
-    static_assert(FA != 1, "pairs along y need an inlet/outlet axis other than y");
-    const int pf = FA == 0 ? x : z;
-    const bool inout = READER && bnd_tile && a.bc[FA] == BC_INOUT;
-    const bool at_in = inout && pf == 0 && !a.cut[0];
-    const bool at_out = inout && pf == (FA == 0 ? g.nx : g.nz) - 1 && !a.cut[1];
+    for (int l = 0; l < 2; ++l) ghosts[l] = BOUNDARY && (l == 0 || has1) && step_writes_ghosts<2>(g, a.bc, x, y + l, 0);
+    const bool inout = BOUNDARY && a.bc[0] == BC_INOUT;
+    const bool at_in = inout && x == 0 && !a.cut[0];
+    const bool at_out = inout && x == g.nx - 1 && !a.cut[1];
 
     // ---- flow: gather (bounce-back and inlet per node), moments, BGK ----
     float2 u[3] = {p_all(0.0f), p_all(0.0f), p_all(0.0f)};
@@ -142,16 +123,16 @@ __device__ __forceinline__ void step_pair(const StepArgs<DIM, ST> &a, int x0, in
         float2 d[F::Q];
 #pragma unroll
         for (int i = 0; i < F::Q; ++i) {
-            const int off = F::c(i, 0) + F::c(i, 1) * g.px + F::c(i, 2) * (int)g.zs;
+            const int off = F::c(i, 0) + F::c(i, 1) * g.px;
             float v[2];
 #pragma unroll
             for (int l = 0; l < 2; ++l) {
                 // bounce-back, or the moving-wall value entering across the inlet
                 const bool bb = i > 0 && ((L[l] >> i) & 1u);
-                const bool inj = F::c(i, FA) == 1 && at_in && !bb;
+                const bool inj = F::c(i, 0) == 1 && at_in && !bb;
                 const int o = (bb || inj) ? F::opp(i) * P : i * P - off;
                 v[l] = ld(a.fsrc + MFC_IDX(k[l] + o, F::Q * P));
-                if (F::c(i, FA) == 1 && inj) v[l] += a.bb_in[i];
+                if (F::c(i, 0) == 1 && inj) v[l] += a.bb_in[i];
             }
             d[i] = make_float2(v[0], v[1]);
         }
@@ -165,22 +146,20 @@ __device__ __forceinline__ void step_pair(const StepArgs<DIM, ST> &a, int x0, in
         const float2 opr = p_add(p_all(1.0f), rp);
         const float2 inv = make_float2(recip(opr.x), recip(opr.y));
 #pragma unroll
-        for (int ax = 0; ax < DIM; ++ax)
+        for (int ax = 0; ax < 2; ++ax)
             u[ax] = p_mul(p_sub(p_sum_where<F>(d, ax, 1), p_sum_where<F>(d, ax, -1)), inv);
-        float2 uu = p_mul(u[0], u[0]);
-#pragma unroll
-        for (int ax = 1; ax < DIM; ++ax) uu = p_fma(u[ax], u[ax], uu);
+        const float2 uu = p_fma(u[1], u[1], p_mul(u[0], u[0]));
         const float2 muu = p_mul(p_all(-1.5f), uu);
         const float2 om = p_all(a.omega);
-        // w (1 + rho') and w rho' of the two moving weight classes (faces; diagonals or edges)
-        constexpr int IE = DIM == 2 ? 5 : 7;
+        // w (1 + rho') and w rho' of the two moving weight classes (faces; diagonals)
+        constexpr int IE = 5;
         const float2 wo_f = p_mul(p_all(F::w(1)), opr), wr_f = p_mul(p_all(F::w(1)), rp);
         const float2 wo_e = p_mul(p_all(F::w(IE)), opr), wr_e = p_mul(p_all(F::w(IE)), rp);
         float2 moved = p_all(0.0f);
 #pragma unroll
         for (int i = 1; i < F::Q; ++i) {
             float s;
-            const float2 m = p_cdot<F, DIM>(i, u, s);
+            const float2 m = p_cdot<F, 2>(i, u, s);
             // 3 cu + 9/2 cu^2 - 3/2 u.u = m (9/2 m + 3 s) - 3/2 u.u
             const float2 t = p_fma(m, p_fma(p_all(4.5f), m, p_all(3.0f * s)), muu);
             const float2 feq = i < IE ? p_fma(wo_f, t, wr_f) : p_fma(wo_e, t, wr_e);
@@ -195,9 +174,7 @@ __device__ __forceinline__ void step_pair(const StepArgs<DIM, ST> &a, int x0, in
             const bool open = l == 0 ? open0 : open1;
             if (!(ghosts[l] && open)) continue;
             const float u0 = l == 0 ? u[0].x : u[0].y, u1 = l == 0 ? u[1].x : u[1].y;
-            const float u2 = l == 0 ? u[2].x : u[2].y;
-            if constexpr (READER) flow_ghosts_step<DIM, ST>(a, a.fdst, x, y + l, z, k[l], u0, u1, u2);
-            else flow_ghosts<DIM, ST>(a, a.fdst, x, y + l, z, k[l], L[l], u0, u1, u2);
+            flow_ghosts_step<2, ST>(a, a.fdst, x, y + l, 0, k[l], u0, u1, 0.0f);
         }
     }
 
@@ -205,21 +182,21 @@ __device__ __forceinline__ void step_pair(const StepArgs<DIM, ST> &a, int x0, in
     {
         const float2 us = p_all(a.u_scale);
 #pragma unroll
-        for (int ax = 0; ax < DIM; ++ax) u[ax] = p_mul(u[ax], us);  // 0 on flow-blocked nodes
+        for (int ax = 0; ax < 2; ++ax) u[ax] = p_mul(u[ax], us);  // 0 on flow-blocked nodes
         float2 e[A::Q];
 #pragma unroll
         for (int i = 0; i < A::Q; ++i) {
-            const int off = A::c(i, 0) + A::c(i, 1) * g.px + A::c(i, 2) * (int)g.zs;
+            const int off = A::c(i, 0) + A::c(i, 1) * g.px;
             float v[2];
 #pragma unroll
             for (int l = 0; l < 2; ++l) {
                 const bool bb = i > 0 && ((L[l] >> (LK::ADE_SELF + i)) & 1u);
-                const bool in_v = A::c(i, FA) == 1 && at_in && !bb;
-                const bool out_v = A::c(i, FA) == -1 && at_out && !bb;
+                const bool in_v = A::c(i, 0) == 1 && at_in && !bb;
+                const bool out_v = A::c(i, 0) == -1 && at_out && !bb;
                 const int o = bb ? A::opp(i) * P : i * P - (out_v ? 0 : off);
                 v[l] = ld(a.gsrc + MFC_IDX(k[l] + o, A::Q * P));
-                if (A::c(i, FA) == 1 && in_v) v[l] = a.gin_dev[i];
-                if (A::c(i, FA) == -1 && out_v && a.ade_dirichlet) v[l] = a.gout_dev[i];
+                if (A::c(i, 0) == 1 && in_v) v[l] = a.gin_dev[i];
+                if (A::c(i, 0) == -1 && out_v && a.ade_dirichlet) v[l] = a.gout_dev[i];
             }
             e[i] = make_float2(v[0], v[1]);
         }
@@ -247,7 +224,7 @@ __device__ __forceinline__ void step_pair(const StepArgs<DIM, ST> &a, int x0, in
 #pragma unroll
         for (int i = 1; i < A::Q; ++i) {
             float s;
-            const float2 m = p_cdot<A, DIM>(i, u, s);
+            const float2 m = p_cdot<A, 2>(i, u, s);
             const float2 geq = p_fma(s > 0.0f ? wc_pos : wc_neg, m, wcp);
             const float2 v = p_sub(p_fma(omc, p_sub(geq, e[i]), e[i]), wsink);
             const float2 vk = p_store(a.gdst + MFC_IDX(i * P + k[0], A::Q * P),
@@ -260,8 +237,7 @@ __device__ __forceinline__ void step_pair(const StepArgs<DIM, ST> &a, int x0, in
         for (int l = 0; l < 2; ++l) {
             const bool open = l == 0 ? open0 : open1;
             if (!(ghosts[l] && open)) continue;
-            if constexpr (READER) ade_ghosts_step<DIM, ST>(a, a.gdst, x, y + l, z, k[l]);
-            else ade_ghosts<DIM, ST>(a, a.gdst, x, y + l, z, k[l], L[l]);
+            ade_ghosts_step<2, ST>(a, a.gdst, x, y + l, 0, k[l]);
         }
     }
 }
@@ -272,23 +248,20 @@ __device__ __forceinline__ void step_pair(const StepArgs<DIM, ST> &a, int x0, in
 // never mix on one lattice.
 // (A loop over several row pairs per thread, loading the next pair's link words ahead, measured
 // slower at every depth tried.)
-template <int DIM, typename ST, int SINK>
-__global__ void __launch_bounds__(256, PAIR_BLOCKS) lbm_pair_kernel(const StepArgs<DIM, ST> a)
+template <typename ST, int SINK>
+__global__ void __launch_bounds__(256, PAIR_BLOCKS) lbm_pair_kernel(const StepArgs<2, ST> a)
 {
     const int x0 = blockIdx.x * blockDim.x;
     const int x = x0 + (int)threadIdx.x;
     if (x >= a.geo.nx) return;
     const int y = 2 * (int)blockIdx.y;
-    static_assert(DIM == 2, "3-D plain steps are lbm_row.cuh's");
-    const int z = 0;
     uint32_t L[2];
-    pair_links(a, x, y, z, L);
+    pair_links(a, x, y, L);
     const int y1 = y + 1 < a.geo.ny ? y + 1 : y;
-    if (tile_on_open_boundary<DIM>(a.geo, a.bc, x0, blockDim.x, y, z) ||
-        tile_on_open_boundary<DIM>(a.geo, a.bc, x0, blockDim.x, y1, z))
-        step_pair<DIM, ST, B_BOUNDARY, SINK>(a, x0, y, z, L);
+    if (tile_on_open_boundary<2>(a.geo, a.bc, x0, blockDim.x, y, 0) || tile_on_open_boundary<2>(a.geo, a.bc, x0, blockDim.x, y1, 0))
+        step_pair<ST, true, SINK>(a, x, y, L);
     else
-        step_pair<DIM, ST, B_INTERIOR, SINK>(a, x0, y, z, L);
+        step_pair<ST, false, SINK>(a, x, y, L);
 }
 
 }  // namespace mfc
