@@ -446,9 +446,9 @@ MFC_API mfc_status mfc_field_sums_noalloc(long long n, int dim, const uint8_t *n
  * Requests are admitted first come, first served, as instance slots and device memory free up
  * (each request's device memory, mfc_lattice_bytes plus the read-back staging when fields are
  * asked for, counts against budget_bytes); admitted instances stay resident on the device and
- * advance together, every lattice of every instance in one launch per step and dimension (a
- * fixed grid of a few blocks per SM walking a tile table of all instances' rows), in CUDA-graph
- * replays of K steps that end with every instance's residual check.  A finished instance
+ * advance together, all instances of a dimension in one launch (a fixed grid of a few blocks per
+ * SM walking a table of their tiles; plain steps of 2-D instances with walls across the flow axis
+ * go several per launch), in CUDA-graph replays of K steps that end with every instance's residual check.  A finished instance
  * (converged, at its step cap, timed out, non-finite or out of range) leaves at the end of its
  * block; its fields are copied to the caller's buffers while the next block runs, and its memory
  * goes back to the batch's pool after that block.  Requests that arrive while a block runs are
@@ -469,7 +469,8 @@ typedef struct {
     size_t budget_bytes;  /* device memory for instances; 0 = 90% of the free memory at create */
     int precision;        /* MFC_FP32 or MFC_FP16_DEV, for every instance (MFC_FP64: MFC_ERR_ARG) */
     int check_every;      /* K (even, >= 2; odd values are rounded up); 0 = chosen by the autotuner */
-    int block;            /* threads per tile: 64, 128 or 256; 0 = chosen by the autotuner */
+    int block;            /* threads per row segment (check steps, 2-D steps that go one at a time): 64, 128
+                             or 256; 0 = chosen by the autotuner */
     int max_instances;    /* instance slots, 1..4096; 0 = 256 */
     void *stream;         /* cudaStream_t, or NULL for a library-owned stream */
 } mfc_batch_opts;

@@ -4,7 +4,7 @@
 //   SCALAR_FORM: the grouping of step_node (lbm_kernels.cuh), including which products the
 //     compiler contracts there (measured by comparing the bits): t = 3 cu + (4.5 cu) cu - 1.5 u.u,
 //     feq = w (rho' + (1 + rho') t), f + omega (feq - f), as chains of fused multiply-adds;
-//   PAIR_FORM: the grouping of step_pair (lbm_pair.cuh), the plain coupled step of FP16 storage.
+//   PAIR_FORM: the grouping of step_pair (lbm_pair.cuh), that of plain coupled steps in FP16 storage.
 #pragma once
 
 #include "lbm_pair.cuh"

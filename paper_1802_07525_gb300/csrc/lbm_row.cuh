@@ -22,11 +22,12 @@ enum : int { ROW_BLOCK = 128 };
 // (64x40x48 6.04 us per step, 6.16 in turn; 97x71x83 in FP16, 60 MB, the same).
 constexpr long long BACK_BYTES = 96ll << 20;
 
-// Resident blocks per SM.  FP32 coupled steps gather both sets before the first collision (102 registers, 5
+// Resident blocks per SM.  FP32 coupled steps gather both sets before the first collision (96 registers, 5
 // blocks: 137.4 us per 256x128x128 step, against 141.3 one set after the other at 8 blocks; the one-node
 // kernel took 140); FP16 ones do better with more warps and one set at a time (99.6 us against 104 with
 // both at 6 blocks; two rows per thread took 108.8), as do flow and transport alone (128x64x96: 30.5 us for
-// the two, against 31.5 at 5 blocks and 33.5 with one node per thread).  Small lattices gain the most, from
+// the two, against 31.5 at 5 blocks and 33.5 with one node per thread).  At 8 blocks FP32 flow alone spills 16
+// bytes (256x128x128 98.9 us per step; at 6, without spills, 101.8), the FP16 batch kernel 32.  Small lattices gain the most, from
 // ghost values written from registers: 24x16x16 10.6 -> 4.6 us, 64x40x48 11.4 -> 5.9.
 template <typename ST, bool COUPLED> struct RowOccupancy {
     static constexpr bool both_sets = COUPLED && sizeof(ST) == 4;

@@ -461,8 +461,9 @@ double best_tile(const mfc_lattice *L, int kind, int most, SweepShape *best)
 
 // Columns of a 3-D sweep of two steps: even column tiles, and as many pieces along z as make the last round
 // of blocks (one per SM) full, counting two turns more than planes for each.  Returns whether it is faster
-// than two one-step launches: a turn takes 1.32 us per step (1.24 to 1.49 over 21 lattices of 64x40x48 to
-// 300x200x150), the row kernel at least 0.0323 ns per node, so from 41000 nodes per turn on.  us per step, march
+// than two one-step launches: a turn takes 1.32 us per step (1.16 to 1.51 over 78 lattices), the row kernel at
+// least 0.0314 ns per node, so from 41000 nodes per turn on: there the lattices measured (41000 to 50000 nodes per
+// turn, porosity 0.6 and 1) take 0.77 to 0.997 of the row kernel's time.  us per step, march
 // against row: 120x120x120 53.3 and 57.4, 200x150x100 93.9 and 98.3, 256x128x128 134.3 and 135.7, 256x256x128
 // 250 and 268; 97x71x83 22.9 and 23.4 (taken as even); below the line, 128x128x128 83 and 70, 128x64x96 34.8
 // and 27.7, 64x40x48 9.8 and 6.0.
