@@ -67,7 +67,7 @@ def _digest(verbose: bool, check_bounds: bool = False) -> str:
 
 
 # The files each step-kernel translation unit compiles from (the TU and the headers it includes).
-KERNEL_TU_FILES = ["lbm_launch.cuh", "mfc_internal.h", "lbm_kernels.cuh", "lbm_lattice.cuh", "lbm_pair.cuh", "lbm_collide.cuh", "lbm_sweep.cuh", "lbm_row.cuh", "lbm_march.cuh"]
+KERNEL_TU_FILES = ["lbm_launch.cuh", "mfc_internal.h", "../../include/mfc.h", "lbm_kernels.cuh", "lbm_lattice.cuh", "lbm_pair.cuh", "lbm_collide.cuh", "lbm_sweep.cuh", "lbm_row.cuh", "lbm_march.cuh"]
 
 
 def kernel_digest(tu: str) -> str:
